@@ -843,6 +843,37 @@ FusedGate remap_gate(const FusedGate &g, uint64_t A, int a)
     return r;
 }
 
+// The launch plan of f's gates (complex64, no timing records): the small-state gates of `lazy` on
+// A's qubits, then the others, each cut into passes and single launches.  Made on the first call of
+// each kind and kept with f (its gates, their order and the small-state set never change).
+int ensure_plan(sv_fused *f, sv_fused::Plan *pl, const std::vector<char> *lazy, uint64_t A, int a)
+{
+    if (pl->ready) return SV_OK;
+    std::vector<const FusedGate *> small, rest;
+    pl->small_gates.clear();
+    pl->small_index.clear();
+    pl->rest_index.clear();
+    for (size_t i = 0; i < f->gates.size(); ++i) {
+        if (lazy && (*lazy)[i]) {
+            pl->small_gates.push_back(remap_gate(f->gates[i], A, a));
+            pl->small_index.push_back((int)i);
+        } else {
+            pl->rest_index.push_back((int)i);
+            rest.push_back(&f->gates[i]);
+        }
+    }
+    for (const FusedGate &g : pl->small_gates) small.push_back(&g);
+    try {
+        plan_passes(small, a, &pl->small);
+        plan_passes(rest, f->n, &pl->rest);
+    } catch (const std::exception &) {
+        set_error("sv_apply_fused_gates: out of host memory for the launch plan");
+        return SV_ENOMEM;
+    }
+    pl->ready = true;
+    return SV_OK;
+}
+
 // Applies every fused gate of f to st.  With `lazy` (one flag per gate, a set closed under the
 // gates' order: no flagged gate shares a qubit with an earlier unflagged one) the flagged gates run
 // first, in order, on the small state of the qubits in A started from basis x (see above), which
@@ -856,6 +887,7 @@ int apply_core(sv_state *st, sv_fused *f, sv_timing *timings, const std::vector<
                 set_error("%s: post-phases and swap networks (SV_FUSE_PHASES) are for complex64 states", who);
                 return SV_EINVAL;
             }
+    std::lock_guard<std::mutex> use(f->mu);
     if (st->c128) SV_TRY(upload_fused_c128(f, st->device));
     else SV_TRY(upload_fused(f, st->device));
     const size_t ng = f->gates.size();
@@ -925,31 +957,54 @@ int apply_core(sv_state *st, sv_fused *f, sv_timing *timings, const std::vector<
                             st->n >= g0.k + 5 && g0.post.empty();
     }
     int rc = SV_OK;
-    for (size_t oi = 0; oi < ng && rc == SV_OK; ++oi) {
-        if (m > 0 && oi == m && !first_reads_small) rc = expand();
-        if (rc != SV_OK) break;
-        const size_t i = order[oi];
-        const bool on_small = oi < m;
+    auto device_mats = [&](size_t i) -> const float * {
+        return (i < f->mat_offset.size() && f->mat_offset[i] != SIZE_MAX) ? f->d_mats + f->mat_offset[i] : nullptr;
+    };
+    auto device_tc = [&](size_t i) -> const void * {
+        return (f->d_tc && i < f->tc_offset.size() && f->tc_offset[i] != SIZE_MAX) ? static_cast<const char *>(f->d_tc) + f->tc_offset[i]
+                                                                                   : nullptr;
+    };
+    auto small_gate = [&](const FusedGate &rg, size_t i) -> int {
+        const bool tc = rg.path == SV_PATH_TC_TF32 || rg.path == SV_PATH_TC_BF16X3;
+        return launch_fused_gate(small, a, rg, device_mats(i), tc ? device_tc(i) : nullptr, st->stream, st->num_sms);
+    };
+    auto full_gate = [&](size_t i) -> int {
         const FusedGate &g = f->gates[i];
-        const float *dm = (i < f->mat_offset.size() && f->mat_offset[i] != SIZE_MAX) ? f->d_mats + f->mat_offset[i] : nullptr;
-        const void *dt = (f->d_tc && i < f->tc_offset.size() && f->tc_offset[i] != SIZE_MAX)
-                             ? static_cast<const char *>(f->d_tc) + f->tc_offset[i] : nullptr;
-        if (timings) cudaEventRecord(ev[2 * i], st->stream);
-        if (on_small) {
-            const FusedGate rg = remap_gate(g, A, a);
-            const bool tc = rg.path == SV_PATH_TC_TF32 || rg.path == SV_PATH_TC_BF16X3;
-            rc = launch_fused_gate(small, a, rg, dm, tc ? dt : nullptr, st->stream, st->num_sms);
-        } else if (st->c128) {
+        if (st->c128) {
             const double *um = (f->d_mats64 && f->mat64_offset[i] != SIZE_MAX) ? f->d_mats64 + f->mat64_offset[i] : nullptr;
-            rc = c128_apply_gate(st, g, um);
-        } else if (first_reads_small && oi == m) {
+            return c128_apply_gate(st, g, um);
+        }
+        if (first_reads_small && i == order[m]) {
             const uint64_t rest = x & ~A & nmask;
             const TcSource vs{small, nmask & ~amask, rest, (long long)((rest >> 5) << 6)};
-            rc = launch_tc_gate(st->d, st->n, g, dt, st->stream, st->num_sms, &vs);
-        } else {
-            rc = launch_fused_gate(st->d, st->n, g, dm, dt, st->stream, st->num_sms);
+            return launch_tc_gate(st->d, st->n, g, device_tc(i), st->stream, st->num_sms, &vs);
         }
-        if (timings) cudaEventRecord(ev[2 * i + 1], st->stream);
+        return launch_fused_gate(st->d, st->n, g, device_mats(i), device_tc(i), st->stream, st->num_sms);
+    };
+    if (!timings && !st->c128) {
+        // no record per gate is asked for: gates go in passes (the plan; see sv_stage.cu)
+        sv_fused::Plan *pl = &f->plans[m > 0 ? 1 : 0];
+        rc = ensure_plan(f, pl, m > 0 ? lazy : nullptr, A, a);
+        for (size_t s = 0; rc == SV_OK && s < pl->small.steps.size(); ++s) {
+            const PassStep &ps = pl->small.steps[s];
+            if (ps.single < 0) rc = launch_stage(small, ps, st->stream, st->num_sms);
+            else rc = small_gate(pl->small_gates[(size_t)ps.single], (size_t)pl->small_index[(size_t)ps.single]);
+        }
+        if (rc == SV_OK && m > 0 && m < ng && !first_reads_small) rc = expand();
+        for (size_t s = 0; rc == SV_OK && s < pl->rest.steps.size(); ++s) {
+            const PassStep &ps = pl->rest.steps[s];
+            if (ps.single < 0) rc = launch_stage(st->d, ps, st->stream, st->num_sms);
+            else rc = full_gate((size_t)pl->rest_index[(size_t)ps.single]);
+        }
+    } else {
+        for (size_t oi = 0; oi < ng && rc == SV_OK; ++oi) {
+            if (m > 0 && oi == m && !first_reads_small) rc = expand();
+            if (rc != SV_OK) break;
+            const size_t i = order[oi];
+            if (timings) cudaEventRecord(ev[2 * i], st->stream);
+            rc = oi < m ? small_gate(remap_gate(f->gates[i], A, a), i) : full_gate(i);
+            if (timings) cudaEventRecord(ev[2 * i + 1], st->stream);
+        }
     }
     if (rc == SV_OK && m > 0 && m == ng) rc = expand();
     if (timings && ng) {

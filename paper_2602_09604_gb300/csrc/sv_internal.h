@@ -120,6 +120,26 @@ int device_sm_count(int device);
 // Swap networks (sv_swap.cu): one in-place pass applying g.swaps (10 <= n qubits).
 int launch_swaps(float *sv, int n, const FusedGate &g, cudaStream_t stream, int num_sms);
 
+// Staged passes (sv_stage.cu): runs of CUDA-core gates applied tile by tile in shared memory, one
+// read and one write of the state per run.
+constexpr int kStageQubits = 12;      // local qubits of a tile (32 KB)
+
+// What one launch does: a pass, or the one gate `single` on its own kernel.
+struct PassStep {
+    int single = -1;
+    int form = 0;               // size class of the pass's matrices
+    long long tiles = 0;
+    std::vector<unsigned long long> args;   // the pass's kernel argument block
+};
+struct PassPlan {
+    std::vector<PassStep> steps;
+};
+// Cuts gates (in circuit order, on an n-qubit state) into passes and single launches.  Gates move
+// ahead only of gates on other qubits, and not at all in a circuit with tensor-core gates (their
+// operand split turns a last-bit difference of the input into a larger one).
+void plan_passes(const std::vector<const FusedGate *> &gates, int n, PassPlan *plan);
+int launch_stage(float *sv, const PassStep &p, cudaStream_t stream, int num_sms);
+
 // Tensor-core path (sv_tc.cu): host-side operand images and the launcher.
 // Tensor-core operand images of f's tensor-core gates: plan_tc_operands sets f->tc_offset (byte
 // offsets, 128-byte aligned) and the total size; write_tc_operands writes every image at
@@ -216,6 +236,16 @@ struct sv_fused {
     double *d_mats64 = nullptr;     // fp64 (re, im) images of k >= 5 gates, for complex128 states
     size_t d_mats64_bytes = 0;
     std::vector<size_t> mat64_offset;
+    // launch plans for the calls without timing records, one for sv_apply_fused_gates and one for
+    // sv_init_apply (made on first use: the gates, their order and the small-state set are fixed)
+    struct Plan {
+        bool ready = false;
+        std::vector<svg::FusedGate> small_gates;   // sv_init_apply: the gates of the small state, renumbered
+        std::vector<int> small_index, rest_index;  // their and the other gates' indices, in order
+        svg::PassPlan small, rest;
+    };
+    Plan plans[2];
+    std::mutex mu;                                 // uploads, plans and use_events
     // one event per stream that has applied this circuit, recorded after its last launch there:
     // sv_fused_free waits for these (not for the whole device) before the images are reused
     std::vector<std::pair<cudaStream_t, cudaEvent_t>> use_events;
