@@ -29,9 +29,11 @@
 // accumulator.
 #include <algorithm>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "sv_internal.h"
+#include "sv_tile.h"
 
 namespace svg {
 namespace {
@@ -276,6 +278,212 @@ int launch_ev(const float *sv, const EvArgs &a, double *partials, unsigned *coun
     return SV_OK;
 }
 
+// ------------------------------------------------------------------------------------ tiles
+// Many strings in one read pass.  The chain Hamiltonians of variational runs hold many strings
+// with different x masks, each a read of the whole state for the kernel above.  Here a CTA keeps a
+// tile -- 2^12 amplitudes agreeing on the qubits outside a local set that holds qubits 0-4 -- in
+// shared memory and evaluates every string whose x mask lies in the local set: per x mask (and
+// component) each thread forms 16 terms, takes their 16-point Walsh-Hadamard transform (every
+// sign pattern a z mask can put on the four index bits that vary in the thread), and each string sums
+// the 128 threads' entries for its mask, signed by its thread-index and tile parities.  z masks may
+// name any qubit.  Terms of a pair (j, j ^ x) are equal once signed, so only one of each pair is formed.
+constexpr int kEvtThreads = 128;
+constexpr int kEvtQubits = 12;
+constexpr int kEvtGroups = 32;
+constexpr int kEvtStrings = 64;
+
+struct EvtGroup {
+    unsigned short xv;        // address XOR to the partner amplitude
+    unsigned short ov[12];    // address vectors: 7 thread bits, 4 bits inside the thread, the round bit (x = 0)
+    unsigned char rounds;     // 2 when x = 0 (2^12 terms), else 1
+    unsigned char comp;       // 0: real part of the term, 1: imaginary part
+    unsigned char s0, s1;     // its strings
+};
+struct EvtString {
+    unsigned long long z_out; // z outside the tile
+    unsigned char zt, zw, zr; // z on the thread bits, the in-thread bits, the round bit
+};
+struct EvtArgs {
+    TileGeom t;
+    long long tiles;
+    int n_groups, n_strings;
+    EvtGroup g[kEvtGroups];
+    EvtString s[kEvtStrings];
+};
+
+__device__ __forceinline__ float pick_sign(float v, unsigned odd) { return __uint_as_float(__float_as_uint(v) ^ (odd << 31)); }
+
+__global__ void __launch_bounds__(kEvtThreads, 3) expval_tile_kernel(const float *__restrict__ sv, const __grid_constant__ EvtArgs a,
+                                                                     double *__restrict__ partials)
+{
+    extern __shared__ __align__(16) float smem[];
+    float *tile = smem;
+    float *red = smem + (64 << a.t.fb);                                   // two buffers of 16 x 128 entries
+    float2 *acc = reinterpret_cast<float2 *>(red + 2 * 16 * kEvtThreads);   // per string and lane
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const TileMover<kEvtThreads> mv(a.t);
+    for (int i = tid; i < a.n_strings * 32; i += kEvtThreads) acc[i] = make_float2(0.f, 0.f);
+    int pb = 0;
+    for (long long t = blockIdx.x; t < a.tiles; t += gridDim.x) {
+        const unsigned long long b0 = tile_base(a.t, (unsigned long long)t);
+        __syncthreads();   // the last tile's readers are done
+        mv.load(a.t, sv + (long long)(b0 << 6), tile);
+        __syncthreads();
+        for (int gi = 0; gi < a.n_groups; ++gi) {
+            const EvtGroup &g = a.g[gi];
+            unsigned bt = 0;
+#pragma unroll
+            for (int b = 0; b < 7; ++b) bt ^= (0u - ((unsigned)(tid >> b) & 1u)) & (unsigned)g.ov[b];
+            for (int r = 0; r < g.rounds; ++r) {
+                const unsigned base = r ? bt ^ g.ov[11] : bt;
+                float w[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    unsigned o = base;
+#pragma unroll
+                    for (int b = 0; b < 4; ++b)
+                        if ((i >> b) & 1) o ^= g.ov[7 + b];
+                    const unsigned p = o ^ g.xv;
+                    const float ur = tile[o], ui = tile[o + 32], vr = tile[p], vi = tile[p + 32];
+                    w[i] = g.comp ? fmaf(vr, ui, -(vi * ur)) : fmaf(vr, ur, vi * ui);
+                }
+#pragma unroll
+                for (int h = 1; h < 16; h <<= 1)
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        if (!(i & h)) {
+                            const float x = w[i], y = w[i + h];
+                            w[i] = x + y;
+                            w[i + h] = x - y;
+                        }
+                float *rb = red + pb * 16 * kEvtThreads;
+#pragma unroll
+                for (int i = 0; i < 16; ++i) rb[i * kEvtThreads + tid] = w[i];
+                __syncthreads();
+                // two buffers: a warp that writes the next one has read this one
+                for (int s = g.s0 + ((warp - g.s0) & 3); s < g.s1; s += 4) {
+                    const EvtString &z = a.s[s];
+                    const unsigned odd = (unsigned)(__popcll((b0 << 5) & z.z_out) & 1) ^ (r ? z.zr : 0u);
+                    float sum = 0.f;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int e = lane + 32 * k;
+                        sum += pick_sign(rb[z.zw * kEvtThreads + e], (unsigned)__popc(e & z.zt) & 1u);
+                    }
+                    const float2 v = acc[s * 32 + lane];
+                    FF2 f{v.x, v.y};
+                    ff_add(f, pick_sign(sum, odd));
+                    acc[s * 32 + lane] = make_float2(f.hi, f.lo);
+                }
+                pb ^= 1;
+            }
+        }
+    }
+    for (int gi = 0; gi < a.n_groups; ++gi)
+        for (int s = a.g[gi].s0 + ((warp - a.g[gi].s0) & 3); s < a.g[gi].s1; s += 4) {
+            const float2 v = acc[s * 32 + lane];
+            const double d = warp_sum((double)v.x + (double)v.y);
+            if (lane == 0) partials[(size_t)blockIdx.x * a.n_strings + s] = a.g[gi].xv ? 2.0 * d : d;
+        }
+}
+
+// one CTA per string: the CTAs' partials in a fixed order
+__global__ void __launch_bounds__(128) expval_sum_kernel(const double *__restrict__ partials, int ctas, int n_strings,
+                                                         double *__restrict__ result)
+{
+    __shared__ double red[4];
+    double s = 0.0;
+    for (int i = threadIdx.x; i < ctas; i += 128) s += partials[(size_t)i * n_strings + blockIdx.x];
+    s = warp_sum(s);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) result[blockIdx.x] = (red[0] + red[1]) + (red[2] + red[3]);
+}
+
+constexpr int kEvtSmem = (8 << kEvtQubits) + 2 * 16 * kEvtThreads * (int)sizeof(float) + kEvtStrings * 32 * (int)sizeof(float2);
+
+// The tile pass of the strings order[..] listed in `runs` (each a run of equal x masks); res[i]
+// receives the i-th string's sum in the order of `placed`.
+struct EvRun {
+    int pos, m;   // order[pos .. pos + m)
+};
+
+void fill_tiles(const std::vector<EvRun> &runs, const std::vector<int> &order, const uint64_t *x_masks, const uint64_t *z_masks, int n,
+                uint64_t lam, EvtArgs *a, std::vector<int> *placed)
+{
+    std::memset(a, 0, sizeof(*a));
+    placed->clear();
+    int local_of[64], L = 0;
+    for (int q = 0; q < n; ++q) {
+        local_of[q] = -1;
+        if ((lam >> q) & 1) local_of[q] = L++;
+    }
+    fill_geom(lam, n, &a->t);
+    a->tiles = 1ll << (n - L);
+    for (const EvRun &run : runs)
+        for (int comp = 0; comp < 2; ++comp) {
+            EvtGroup &g = a->g[a->n_groups];
+            const uint64_t x = x_masks[order[(size_t)run.pos]];
+            g.s0 = (unsigned char)placed->size();
+            int top = -1;
+            g.xv = 0;
+            for (int q = 0; q < n; ++q)
+                if ((x >> q) & 1) {
+                    g.xv = (unsigned short)(g.xv ^ addr_vec(local_of[q]));
+                    top = local_of[q];
+                }
+            std::vector<int> free_bits, ob;
+            for (int t = 0; t < L; ++t)
+                if (t != top) free_bits.push_back(t);
+            lane_bits(free_bits, &ob);
+            for (size_t b = 0; b < ob.size(); ++b) g.ov[b] = (unsigned short)addr_vec(ob[b]);
+            g.rounds = x ? 1 : 2;
+            g.comp = (unsigned char)comp;
+            for (int i = 0; i < run.m; ++i) {
+                const int s = order[(size_t)(run.pos + i)];
+                const uint64_t z = z_masks[s];
+                if ((__builtin_popcountll(x & z) & 1) != comp) continue;
+                EvtString &o = a->s[placed->size()];
+                o.z_out = z & ~lam;
+                unsigned bits = 0;   // z on the ordered index bits
+                for (size_t b = 0; b < ob.size(); ++b)
+                    for (int q = 0; q < n; ++q)
+                        if (local_of[q] == ob[b] && ((z >> q) & 1)) bits |= 1u << b;
+                o.zt = (unsigned char)(bits & 127u);
+                o.zw = (unsigned char)((bits >> 7) & 15u);
+                o.zr = (unsigned char)((bits >> 11) & 1u);
+                placed->push_back(s);
+            }
+            g.s1 = (unsigned char)placed->size();
+            if (g.s1 > g.s0) ++a->n_groups;
+        }
+    a->n_strings = (int)placed->size();
+}
+
+std::mutex g_evt_mu;
+uint64_t g_evt_attr = 0;
+
+int launch_tiles(const float *sv, const EvtArgs &a, double *partials, double *result, int num_sms, cudaStream_t s)
+{
+    int dev = 0;
+    SV_CUDA_TRY(cudaGetDevice(&dev));
+    const uint64_t bit = dev >= 0 && dev < 64 ? (1ull << dev) : 0ull;
+    {
+        std::lock_guard<std::mutex> lk(g_evt_mu);
+        if (!(g_evt_attr & bit) || !bit) {
+            SV_CUDA_TRY(cudaFuncSetAttribute(expval_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kEvtSmem));
+            g_evt_attr |= bit;
+        }
+    }
+    const int grid = (int)std::min<long long>(a.tiles, 3ll * num_sms);
+    const int smem = (int)sizeof(float) * (64 << a.t.fb) + 2 * 16 * kEvtThreads * (int)sizeof(float) + a.n_strings * 32 * (int)sizeof(float2);
+    expval_tile_kernel<<<grid, kEvtThreads, smem, s>>>(sv, a, partials);
+    SV_CUDA_TRY(cudaGetLastError());
+    expval_sum_kernel<<<a.n_strings, 128, 0, s>>>(partials, grid, a.n_strings, result);
+    SV_CUDA_TRY(cudaGetLastError());
+    return SV_OK;
+}
+
 int highest_bit(unsigned long long v)
 {
     int h = -1;
@@ -307,19 +515,20 @@ extern "C" int sv_expval_pauli(const sv_state *st_c, const uint64_t *x_masks, co
         }
     // workspace: per-CTA partials for one launch, a counter, and one result per string
     const int max_grid = st->num_sms * 8;
+    const size_t n_partials = (size_t)st->num_sms * std::max(8 * kEvMaxStrings, 3 * kEvtStrings);
     if (count > st->ev_capacity) {
         cudaStreamSynchronize(st->stream);
         cudaFree(st->d_ev);
         st->d_ev = nullptr;
         st->ev_capacity = 0;
-        const size_t doubles = (size_t)max_grid * kEvMaxStrings + (size_t)count + 1;
+        const size_t doubles = n_partials + (size_t)count + 1;
         cudaError_t e = cudaMalloc(&st->d_ev, sizeof(double) * doubles);
         if (e == cudaSuccess) e = cudaMemsetAsync(st->d_ev, 0, sizeof(double) * doubles, st->stream);
         if (e != cudaSuccess) { set_error("sv_expval_pauli: workspace allocation failed: %s", cudaGetErrorString(e)); return SV_ENOMEM; }
         st->ev_capacity = count;
     }
     double *partials = st->d_ev;
-    double *results = partials + (size_t)max_grid * kEvMaxStrings;
+    double *results = partials + n_partials;
     unsigned *counter = reinterpret_cast<unsigned *>(results + st->ev_capacity);
 
     // strings grouped by x mask (first-appearance order), at most kEvMaxStrings per pass
@@ -328,11 +537,57 @@ extern "C" int sv_expval_pauli(const sv_state *st_c, const uint64_t *x_masks, co
     std::stable_sort(order.begin(), order.end(), [&](int p, int q) { return x_masks[p] < x_masks[q]; });
     const long long nb = n >= 5 ? (1ll << (n - 5)) : 1ll;
     std::vector<int> slot_of((size_t)count);
-    int pos = 0;
-    while (pos < count) {
-        const uint64_t x = x_masks[order[(size_t)pos]];
+    int out_pos = 0;   // next slot of `results`
+    // Runs of equal x masks (cut at half a tile pass's strings).  Runs whose masks fit one tile's local
+    // qubits share a read of the state; a tile pass is taken when it replaces two or more passes of the
+    // kernel above (its own work per string is larger, so one pass alone is better left there).
+    std::vector<EvRun> runs, left;
+    for (int p = 0; p < count;) {
         int m = 0;
-        while (pos + m < count && m < kEvMaxStrings && x_masks[order[(size_t)(pos + m)]] == x) ++m;
+        while (p + m < count && m < kEvtStrings / 2 && x_masks[order[(size_t)(p + m)]] == x_masks[order[(size_t)p]]) ++m;
+        runs.push_back(EvRun{p, m});
+        p += m;
+    }
+    if (n >= kEvtQubits) {
+        while (!runs.empty()) {
+            uint64_t lam = 31;
+            int strings = 0, passes = 0;
+            std::vector<EvRun> took, rest;
+            for (const EvRun &r : runs) {
+                const uint64_t with = lam | x_masks[order[(size_t)r.pos]];
+                if (__builtin_popcountll(with) <= kEvtQubits && strings + r.m <= kEvtStrings && 2 * (took.size() + 1) <= kEvtGroups) {
+                    lam = with;
+                    strings += r.m;
+                    passes += (r.m + kEvMaxStrings - 1) / kEvMaxStrings;
+                    took.push_back(r);
+                } else {
+                    rest.push_back(r);
+                }
+            }
+            if (took.empty()) {   // the first run's mask fits no tile
+                left.push_back(runs.front());
+                runs.erase(runs.begin());
+                continue;
+            }
+            if (passes < 2) {
+                left.insert(left.end(), took.begin(), took.end());
+            } else {
+                for (int q = 5; q < n && __builtin_popcountll(lam) < kEvtQubits; ++q) lam |= uint64_t(1) << q;
+                EvtArgs a;
+                std::vector<int> placed;
+                fill_tiles(took, order, x_masks, z_masks, n, lam, &a, &placed);
+                SV_TRY(launch_tiles(st->d, a, partials, results + out_pos, st->num_sms, st->stream));
+                for (int s : placed) slot_of[(size_t)s] = out_pos++;
+            }
+            runs.swap(rest);
+        }
+    } else {
+        left.swap(runs);
+    }
+    for (const EvRun &run : left)
+    for (int pos = run.pos; pos < run.pos + run.m;) {
+        const uint64_t x = x_masks[order[(size_t)pos]];
+        const int m = std::min(kEvMaxStrings, run.pos + run.m - pos);
         EvArgs a;
         std::memset(&a, 0, sizeof(a));
         a.xb = x >> 5;
@@ -356,12 +611,12 @@ extern "C" int sv_expval_pauli(const sv_state *st_c, const uint64_t *x_masks, co
             a.zl[p] = (unsigned)(z_masks[s] & 31u);
             a.pairpar[p] = (unsigned)(__builtin_popcountll(a.xb & zb) & 1);
             a.comp[p] = __builtin_popcountll(x & z_masks[s]) & 1;
-            slot_of[(size_t)s] = pos + p;
+            slot_of[(size_t)s] = out_pos + p;
         }
         const long long ranges = (a.n_units + kEvRange - 1) / kEvRange;
         const long long work = (ranges * 32 + kEvThreads - 1) / kEvThreads;   // CTAs with a range per warp
         const float *sv = st->d;
-        double *res = results + pos;
+        double *res = results + out_pos;
         int rc;
         if (m == 1) rc = launch_ev<1>(sv, a, partials, counter, res, work, st->num_sms, max_grid, st->stream);
         else if (m == 2) rc = launch_ev<2>(sv, a, partials, counter, res, work, st->num_sms, max_grid, st->stream);
@@ -369,6 +624,7 @@ extern "C" int sv_expval_pauli(const sv_state *st_c, const uint64_t *x_masks, co
         else rc = launch_ev<8>(sv, a, partials, counter, res, work, st->num_sms, max_grid, st->stream);
         if (rc != SV_OK) return rc;
         pos += m;
+        out_pos += m;
     }
     std::vector<double> host((size_t)count + kEvMaxStrings);
     SV_CUDA_TRY(cudaMemcpyAsync(host.data(), results, sizeof(double) * (size_t)count, cudaMemcpyDeviceToHost, st->stream));
