@@ -844,9 +844,10 @@ FusedGate remap_gate(const FusedGate &g, uint64_t A, int a)
 }
 
 // The launch plan of f's gates (complex64, no timing records): the small-state gates of `lazy` on
-// A's qubits, then the others, each cut into passes and single launches.  Made on the first call of
-// each kind and kept with f (its gates, their order and the small-state set never change).
-int ensure_plan(sv_fused *f, sv_fused::Plan *pl, const std::vector<char> *lazy, uint64_t A, int a)
+// A's qubits, then the others, each cut into passes and single launches; the passes' descriptors and
+// matrices go to one device buffer.  Made on the first call of each kind and kept with f (its gates,
+// their order and the small-state set never change).
+int ensure_plan(sv_fused *f, sv_fused::Plan *pl, const std::vector<char> *lazy, uint64_t A, int a, int device)
 {
     if (pl->ready) return SV_OK;
     std::vector<const FusedGate *> small, rest;
@@ -869,6 +870,34 @@ int ensure_plan(sv_fused *f, sv_fused::Plan *pl, const std::vector<char> *lazy, 
     } catch (const std::exception &) {
         set_error("sv_apply_fused_gates: out of host memory for the launch plan");
         return SV_ENOMEM;
+    }
+    const size_t ns = pl->small.image.size(), nr = pl->rest.image.size();
+    pl->rest_off = ns;
+    const size_t bytes = (ns + nr) * sizeof(float);
+    if (bytes > 0) {
+        void *buf = nullptr;
+        size_t got = 0;
+        SV_TRY(dev_buffer_get(device, bytes, &buf, &got));
+        std::unique_lock<std::mutex> lk;
+        unsigned char *img = nullptr;
+        int rc = pinned_staging(bytes, &img, lk);
+        if (rc == SV_OK) {
+            if (ns) std::memcpy(img, pl->small.image.data(), ns * sizeof(float));
+            if (nr) std::memcpy(img + ns * sizeof(float), pl->rest.image.data(), nr * sizeof(float));
+            const cudaError_t e = cudaMemcpy(buf, img, bytes, cudaMemcpyHostToDevice);
+            if (e != cudaSuccess) {
+                set_error("sv_apply_fused_gates: pass images: %s", cudaGetErrorString(e));
+                rc = SV_ECUDA;
+            }
+        }
+        if (rc != SV_OK) {
+            dev_buffer_put(device, buf, got);
+            return rc;
+        }
+        pl->d_plan = static_cast<float *>(buf);
+        pl->d_plan_bytes = got;
+        pl->small.image = std::vector<float>();
+        pl->rest.image = std::vector<float>();
     }
     pl->ready = true;
     return SV_OK;
@@ -984,16 +1013,16 @@ int apply_core(sv_state *st, sv_fused *f, sv_timing *timings, const std::vector<
     if (!timings && !st->c128) {
         // no record per gate is asked for: gates go in passes (the plan; see sv_stage.cu)
         sv_fused::Plan *pl = &f->plans[m > 0 ? 1 : 0];
-        rc = ensure_plan(f, pl, m > 0 ? lazy : nullptr, A, a);
+        rc = ensure_plan(f, pl, m > 0 ? lazy : nullptr, A, a, st->device);
         for (size_t s = 0; rc == SV_OK && s < pl->small.steps.size(); ++s) {
             const PassStep &ps = pl->small.steps[s];
-            if (ps.single < 0) rc = launch_stage(small, ps, st->stream, st->num_sms);
+            if (ps.single < 0) rc = launch_stage(small, pl->d_plan, ps, st->stream, st->num_sms);
             else rc = small_gate(pl->small_gates[(size_t)ps.single], (size_t)pl->small_index[(size_t)ps.single]);
         }
         if (rc == SV_OK && m > 0 && m < ng && !first_reads_small) rc = expand();
         for (size_t s = 0; rc == SV_OK && s < pl->rest.steps.size(); ++s) {
             const PassStep &ps = pl->rest.steps[s];
-            if (ps.single < 0) rc = launch_stage(st->d, ps, st->stream, st->num_sms);
+            if (ps.single < 0) rc = launch_stage(st->d, pl->d_plan + pl->rest_off, ps, st->stream, st->num_sms);
             else rc = full_gate((size_t)pl->rest_index[(size_t)ps.single]);
         }
     } else {
@@ -1108,6 +1137,7 @@ extern "C" void sv_fused_free(sv_fused *f)
         f->use_events.clear();
         dev_buffer_put(f->device, f->d_buf, f->d_buf_bytes);
         dev_buffer_put(f->device, f->d_mats64, f->d_mats64_bytes);
+        for (sv_fused::Plan &p : f->plans) dev_buffer_put(f->device, p.d_plan, p.d_plan_bytes);
         if (f->device >= 0 && cur >= 0 && cur != f->device) cudaSetDevice(cur);
     }
     delete f;

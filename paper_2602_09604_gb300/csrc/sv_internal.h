@@ -127,18 +127,20 @@ constexpr int kStageQubits = 12;      // local qubits of a tile (32 KB)
 // What one launch does: a pass, or the one gate `single` on its own kernel.
 struct PassStep {
     int single = -1;
-    int form = 0;               // size class of the pass's matrices
+    int kmax = 0;               // largest gate of the pass
     long long tiles = 0;
-    std::vector<unsigned long long> args;   // the pass's kernel argument block
+    std::vector<unsigned long long> args;   // the pass's kernel arguments
+    size_t image_off = 0;       // its descriptors and matrices: floats into PassPlan::image
 };
 struct PassPlan {
     std::vector<PassStep> steps;
+    std::vector<float> image;   // the passes' descriptors and matrices (16-byte multiples), one after another
 };
 // Cuts gates (in circuit order, on an n-qubit state) into passes and single launches.  Gates move
 // ahead only of gates on other qubits, and not at all in a circuit with tensor-core gates (their
 // operand split turns a last-bit difference of the input into a larger one).
 void plan_passes(const std::vector<const FusedGate *> &gates, int n, PassPlan *plan);
-int launch_stage(float *sv, const PassStep &p, cudaStream_t stream, int num_sms);
+int launch_stage(float *sv, const float *image, const PassStep &p, cudaStream_t stream, int num_sms);
 
 // Tensor-core path (sv_tc.cu): host-side operand images and the launcher.
 // Tensor-core operand images of f's tensor-core gates: plan_tc_operands sets f->tc_offset (byte
@@ -243,6 +245,9 @@ struct sv_fused {
         std::vector<svg::FusedGate> small_gates;   // sv_init_apply: the gates of the small state, renumbered
         std::vector<int> small_index, rest_index;  // their and the other gates' indices, in order
         svg::PassPlan small, rest;
+        size_t rest_off = 0;                       // floats into d_plan of the second part's image
+        float *d_plan = nullptr;                   // both images (released with the circuit)
+        size_t d_plan_bytes = 0;
     };
     Plan plans[2];
     std::mutex mu;                                 // uploads, plans and use_events

@@ -15,11 +15,10 @@
 //
 // What bounds a pass: shared memory moves 2 x 8 bytes an amplitude and gate and the FMA pipe
 // 4 * 2^k multiply-adds an amplitude and gate.  The multiply-adds are issued as packed pairs
-// (fma.rn.f32x2, two rows of one column); the matrices travel in the kernel's parameter block and are
-// read through the constant bank at a run-time, warp-uniform index.  A loop of this form (k = 4, two
-// groups a thread) measured 33.6 T multiply-adds/s on 152 SMs, against 28.4 with the matrices in
-// shared memory (a broadcast 16-byte read costs two passes of the shared-memory pipe) and 24-29 with
-// scalar multiply-adds.
+// (fma.rn.f32x2, two rows of one column).  The pass's descriptors and matrices are copied to shared
+// memory ahead of the tile and read there by broadcast 16-byte loads, each of which costs two passes of
+// the shared-memory pipe: a thread therefore takes four groups at a time for k <= 3 and two for k = 4,
+// so that one such load serves 8 to 16 packed multiply-adds.
 #include <algorithm>
 #include <cstring>
 #include <mutex>
@@ -31,24 +30,24 @@ namespace svg {
 namespace {
 
 // One gate of a pass.  Tile addresses are float offsets, linear over GF(2) in the tile's index bits.
-struct StageGate {
-    uint64_t cm_out;            // control qubits outside the tile: the gate applies to tiles with all of them 1
+struct alignas(16) StageGate {
+    // address vectors of the group-index bits that come from the thread index, two to a word: bit b
+    // in the low half of word b, bit b + 5 in the high half
+    unsigned lane[5];
+    unsigned short step[7];     // address vectors of group-index bits 5-11 (those past the thread index count trips)
+    unsigned short pad;
     unsigned short tv[5];       // address vector of target b
-    unsigned short gv[kStageQubits];   // address vector of group-index bit b (0 from nb on)
     unsigned short cset;        // address of the control bits inside the tile, all 1
     unsigned short moff;        // matrix offset (16-byte units) in the pass's matrices
     unsigned char k, nb;        // targets; group-index bits
+    uint64_t cm_out;            // control qubits outside the tile: the gate applies to tiles with all of them 1
 };
+static_assert(sizeof(StageGate) == 64, "a gate's descriptor is read as 16-byte words");
 constexpr int kStageMaxGates = 48;
-struct alignas(16) StageHead {
+struct StageArgs {
     TileGeom t;
     int n_gates;
-    StageGate g[kStageMaxGates];
-};
-template <int M>
-struct StageArgs {
-    StageHead h;
-    float mat[M];
+    int units;                  // 16-byte units of the pass's image: descriptors, then matrices
 };
 
 typedef unsigned long long f32x2;
@@ -62,119 +61,176 @@ __device__ __forceinline__ f32x2 dup2(float x)
 __device__ __forceinline__ void fma2(f32x2 &d, f32x2 a, f32x2 b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b)); }
 __device__ __forceinline__ void unpack2(f32x2 v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
 
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)   // a * b + 0: the first step of a chain
+{
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(0ull));
+    return d;
+}
+
+// The thread index's bits as masks, laid out as StageGate::lane.
+struct ThreadMasks {
+    unsigned m[5];
+    __device__ __forceinline__ ThreadMasks()
+    {
+#pragma unroll
+        for (int b = 0; b < 5; ++b)
+            m[b] = ((threadIdx.x >> b) & 1u ? 0xffffu : 0u) | ((threadIdx.x >> (b + 5)) & 1u ? 0xffff0000u : 0u);
+    }
+};
+
 // One gate on the tile: a thread takes V groups (group index bits -> tile address by the XOR of the
-// set bits' vectors), accumulates all rows while the columns stream from shared memory, then writes
-// the rows back.  m: column j, row pair p at m[j * D / 2 + p] = (re, re', im, im').
+// set bits' vectors) at a time, accumulates all rows while the columns stream from shared memory, then
+// writes the rows back.  m: column j, row pair p at m[j * D / 2 + p] = (re, re', im, im').
 template <int K, int V, int T>
-__device__ __forceinline__ void stage_gate(float *__restrict__ tile, const ulonglong2 *__restrict__ m, const StageGate &g)
+__device__ __forceinline__ void stage_gate(float *__restrict__ tile, const ulonglong2 *__restrict__ m, const StageGate &g, const ThreadMasks &tm)
 {
     constexpr int D = 1 << K;
     constexpr int LT = T == 128 ? 7 : 9;
-    static_assert((1 << LT) == T, "thread count");
-    const int np = (V == 2 && g.nb > 0) ? g.nb - 1 : g.nb;
-    const unsigned pv = (V == 2 && g.nb > 0) ? g.gv[np] : 0u;
-    unsigned bt = g.cset;
+    constexpr int LV = V == 4 ? 2 : V == 2 ? 1 : 0;
+    static_assert((T == 128 || T == 512) && (1 << LV) == V, "thread and group counts");
+    const int nb = g.nb;
+    // group index = thread index + (trip V + v) T, v < V; a gate with fewer groups than that (kept
+    // controls) repeats its last ones under v: their address bits are 0, and every copy of a group is
+    // read before any is written (one thread holds them all)
+    const bool active = nb >= LT || (threadIdx.x >> nb) == 0;
+    if (active) {
+        unsigned bt = 0;
 #pragma unroll
-    for (int b = 0; b < LT; ++b) bt ^= (0u - ((threadIdx.x >> b) & 1u)) & (unsigned)g.gv[b];
-    if (np < LT && (threadIdx.x >> np) != 0) return;
-    const int iters = np > LT ? 1 << (np - LT) : 1;
-    for (int it = 0; it < iters; ++it) {
-        unsigned base = bt;
-        for (int b = LT; b < np; ++b) base ^= (0u - ((unsigned)(it >> (b - LT)) & 1u)) & (unsigned)g.gv[b];
-        f32x2 yr[V][D / 2], yi[V][D / 2];
+        for (int b = 0; b < 5; ++b) bt ^= tm.m[b] & g.lane[b];
+        bt = (bt & 0xffffu) ^ (bt >> 16) ^ g.cset;
+        unsigned tv[K], pv[V];
 #pragma unroll
-        for (int v = 0; v < V; ++v)
+        for (int b = 0; b < K; ++b) tv[b] = g.tv[b];
 #pragma unroll
-            for (int p = 0; p < D / 2; ++p) yr[v][p] = yi[v][p] = 0ull;
-        // columns in fours, the fours in a real loop: unrolled whole, the compiler keeps every
-        // column's address and operands alive and spills
-        constexpr int JU = D < 4 ? D : 4;
+        for (int v = 0; v < V; ++v) {
+            pv[v] = 0u;
+#pragma unroll
+            for (int b = 0; b < LV; ++b)
+                if ((v >> b) & 1) pv[v] ^= g.step[LT - 5 + b];   // 0 from group-index bit nb on
+        }
+        const int iters = nb > LT + LV ? 1 << (nb - LT - LV) : 1;
 #pragma unroll 1
-        for (int jh = 0; jh < D / JU; ++jh) {
-            unsigned oh = base;
+        for (int it = 0; it < iters; ++it) {
+            unsigned base = bt;
+            for (int b = LT + LV; b < nb; ++b) base ^= ((it >> (b - LT - LV)) & 1) ? (unsigned)g.step[b - 5] : 0u;
+            f32x2 yr[V][D / 2], yi[V][D / 2];
 #pragma unroll
-            for (int b = 2; b < K; ++b) oh ^= ((jh >> (b - 2)) & 1) ? (unsigned)g.tv[b] : 0u;
-            const ulonglong2 *mj = m + jh * (JU * D / 2);
+            for (int v = 0; v < V; ++v)
 #pragma unroll
-            for (int jl = 0; jl < JU; ++jl) {
-                unsigned o = oh;
-                if (jl & 1) o ^= g.tv[0];
-                if (jl & 2) o ^= g.tv[1];
-                f32x2 xr[V], xi[V], xn[V];
+                for (int p = 0; p < D / 2; ++p) yr[v][p] = yi[v][p] = 0ull;   // dead when K <= 2
+            // columns in fours, the fours in a real loop: unrolled whole, the compiler keeps every
+            // column's address and operands alive and spills
+            constexpr int LJ = K < 2 ? K : 2, JU = 1 << LJ;
+#pragma unroll 1
+            for (int jh = 0; jh < D / JU; ++jh) {
+                unsigned oh = base;
 #pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    const unsigned a = v ? o ^ pv : o;
-                    const float r = tile[a], i = tile[a + 32];
-                    xr[v] = dup2(r);
-                    xi[v] = dup2(i);
-                    xn[v] = dup2(-i);
-                }
+                for (int b = LJ; b < K; ++b) oh ^= ((jh >> (b - LJ)) & 1) ? tv[b] : 0u;
+                const ulonglong2 *mj = m + jh * (JU * D / 2);
 #pragma unroll
-                for (int p = 0; p < D / 2; ++p) {
-                    const ulonglong2 u = mj[jl * (D / 2) + p];
+                for (int jl = 0; jl < JU; ++jl) {
+                    unsigned o = oh;
+#pragma unroll
+                    for (int b = 0; b < LJ; ++b)
+                        if ((jl >> b) & 1) o ^= tv[b];
+                    f32x2 xr[V], xi[V], xn[V];
 #pragma unroll
                     for (int v = 0; v < V; ++v) {
-                        fma2(yr[v][p], u.x, xr[v]);
-                        fma2(yr[v][p], u.y, xn[v]);
-                        fma2(yi[v][p], u.x, xi[v]);
-                        fma2(yi[v][p], u.y, xr[v]);
+                        const unsigned a = o ^ pv[v];
+                        const float r = tile[a], i = tile[a + 32];
+                        xr[v] = dup2(r);
+                        xi[v] = dup2(i);
+                        xn[v] = dup2(-i);
+                    }
+#pragma unroll
+                    for (int p = 0; p < D / 2; ++p) {
+                        const ulonglong2 u = mj[jl * (D / 2) + p];
+#pragma unroll
+                        for (int v = 0; v < V; ++v) {
+                            if (K <= 2 && jl == 0) {   // one trip: the chains start here
+                                yr[v][p] = mul2(u.x, xr[v]);
+                                yi[v][p] = mul2(u.x, xi[v]);
+                            } else {
+                                fma2(yr[v][p], u.x, xr[v]);
+                                fma2(yi[v][p], u.x, xi[v]);
+                            }
+                            fma2(yr[v][p], u.y, xn[v]);
+                            fma2(yi[v][p], u.y, xr[v]);
+                        }
                     }
                 }
             }
-        }
 #pragma unroll
-        for (int p = 0; p < D / 2; ++p) {
-            unsigned o = base;
+            for (int p = 0; p < D / 2; ++p) {
+                unsigned o = base;
 #pragma unroll
-            for (int b = 1; b < K; ++b)
-                if ((p >> (b - 1)) & 1) o ^= g.tv[b];
+                for (int b = 1; b < K; ++b)
+                    if ((p >> (b - 1)) & 1) o ^= tv[b];
 #pragma unroll
-            for (int v = 0; v < V; ++v) {
-                const unsigned a = v ? o ^ pv : o;
-                float r0, r1, i0, i1;
-                unpack2(yr[v][p], r0, r1);
-                unpack2(yi[v][p], i0, i1);
-                tile[a] = r0;
-                tile[a + 32] = i0;
-                tile[a ^ g.tv[0]] = r1;
-                tile[(a ^ g.tv[0]) + 32] = i1;
+                for (int v = 0; v < V; ++v) {
+                    const unsigned a = o ^ pv[v];
+                    float r0, r1, i0, i1;
+                    unpack2(yr[v][p], r0, r1);
+                    unpack2(yi[v][p], i0, i1);
+                    tile[a] = r0;
+                    tile[a + 32] = i0;
+                    tile[a ^ tv[0]] = r1;
+                    tile[(a ^ tv[0]) + 32] = i1;
+                }
             }
         }
     }
 }
 
-// T threads a CTA, V groups a thread, matrices of up to M floats (see launch_stage for the forms).
-template <int T, int V, int M>
-__global__ void __launch_bounds__(T, T == 128 ? 5 : 1) stage_kernel(float *__restrict__ sv, const __grid_constant__ StageArgs<M> a)
+// CTAs per SM of the 128-thread form by the largest gate of the pass: what its registers allow without
+// spills that count (28 qubits, 8 cycles, gates of 3: 20.9 ms so; two groups a thread in six CTAs 21.2).
+__host__ __device__ constexpr int stage_ctas(int kmax) { return kmax <= 2 ? 5 : kmax <= 4 ? 4 : 3; }
+
+// T threads a CTA, gates of up to KMAX qubits (see launch_stage for the forms).  A kernel per largest
+// gate: passes of small gates keep their own register count, so more CTAs share an SM.
+template <int T, int KMAX>
+__global__ void __launch_bounds__(T, T == 128 ? stage_ctas(KMAX) : 1) stage_kernel(float *__restrict__ sv, const uint4 *__restrict__ image,
+                                                                                 const __grid_constant__ StageArgs a)
 {
     extern __shared__ __align__(16) float tile[];
-    const TileMover<T> mv(a.h.t);
-    const unsigned long long b0 = tile_base(a.h.t, blockIdx.x);
+    // The pass after this one may start its own set-up; the state is read once the one before is done.
+    asm volatile("griddepcontrol.launch_dependents;");
+    uint4 *img = reinterpret_cast<uint4 *>(tile + (64 << a.t.fb));
+    for (int i = threadIdx.x; i < a.units; i += T) img[i] = __ldg(image + i);
+    const TileMover<T> mv(a.t);
+    const ThreadMasks tm;
+    const unsigned long long b0 = tile_base(a.t, blockIdx.x);
     float *g0 = sv + (long long)(b0 << 6);
-    mv.load(a.h.t, g0, tile);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    mv.load(a.t, g0, tile);
     __syncthreads();
-    for (int i = 0; i < a.h.n_gates; ++i) {
-        const StageGate &g = a.h.g[i];
+    constexpr bool F = T == 512;   // few tiles: one group at a time, so that more threads have one
+    for (int i = 0; i < a.n_gates; ++i) {
+        const StageGate &g = reinterpret_cast<const StageGate *>(img)[i];
         if (((b0 << 5) & g.cm_out) == g.cm_out) {
-            const ulonglong2 *m = reinterpret_cast<const ulonglong2 *>(a.mat + 4 * g.moff);
-            switch (g.k) {
-            case 1: stage_gate<1, V, T>(tile, m, g); break;
-            case 2: stage_gate<2, V, T>(tile, m, g); break;
-            case 3: stage_gate<3, V, T>(tile, m, g); break;
-            case 4: stage_gate<4, V, T>(tile, m, g); break;
-            default: stage_gate<5, 1, T>(tile, m, g); break;
+            const ulonglong2 *m = reinterpret_cast<const ulonglong2 *>(img + g.moff);
+            const int k = g.k;
+            if (k == 1) {
+                stage_gate<1, F ? 1 : 4, T>(tile, m, g, tm);
+            } else if (KMAX <= 2 || k == 2) {
+                stage_gate<2, F ? 1 : 4, T>(tile, m, g, tm);
+            } else if constexpr (KMAX >= 3) {
+                if (KMAX == 3 || k == 3) {
+                    stage_gate<3, F ? 1 : 4, T>(tile, m, g, tm);
+                } else if constexpr (KMAX >= 4) {
+                    if (KMAX == 4 || k == 4) stage_gate<4, F ? 1 : 2, T>(tile, m, g, tm);
+                    else if constexpr (KMAX == 5) stage_gate<5, 1, T>(tile, m, g, tm);
+                }
             }
         }
         __syncthreads();
     }
-    mv.store(a.h.t, tile, g0);
+    mv.store(a.t, tile, g0);
 }
 
 // ------------------------------------------------------------------------------------ planner
-// Matrix space of one pass, in the three parameter-block sizes a launch chooses from (a block is
-// copied by every launch, so short passes take a short one; the limit is 32,764 bytes).
-constexpr int kStageMat[3] = {1024, 2560, 6656};
-constexpr int kStageMatFloats = kStageMat[2];
+constexpr int kStageMatFloats = 4096;   // matrices of one pass: 16 KB, so that four CTAs share an SM
 
 bool stageable(const FusedGate &g)
 {
@@ -193,8 +249,8 @@ uint64_t named(const FusedGate &g)
 size_t mat_floats(const FusedGate &g) { return size_t(2) << (2 * g.k); }
 
 // the launch arguments of a pass over gates `idx` with the local qubits `lam` (bits 0-4 set)
-void fill_stage(const std::vector<const FusedGate *> &gates, const std::vector<int> &idx, uint64_t lam, int n, StageHead *a,
-                float *mat)
+void fill_stage(const std::vector<const FusedGate *> &gates, const std::vector<int> &idx, uint64_t lam, int n, StageArgs *a,
+                std::vector<float> *image)
 {
     std::memset(a, 0, sizeof(*a));
     int local_of[64];
@@ -203,10 +259,13 @@ void fill_stage(const std::vector<const FusedGate *> &gates, const std::vector<i
         if ((lam >> q) & 1) local_of[q] = L++;
     fill_geom(lam, n, &a->t);
     a->n_gates = (int)idx.size();
-    size_t at = 0;
+    constexpr size_t kGateFloats = sizeof(StageGate) / sizeof(float);
+    const size_t at0 = image->size();
+    image->resize(at0 + idx.size() * kGateFloats);
     for (size_t s = 0; s < idx.size(); ++s) {
         const FusedGate &g = *gates[(size_t)idx[s]];
-        StageGate &o = a->g[s];
+        StageGate o;
+        std::memset(&o, 0, sizeof(o));
         o.k = (unsigned char)g.k;
         uint64_t used = 0;   // local bits that are targets or controls
         for (int b = 0; b < g.k; ++b) {
@@ -227,18 +286,24 @@ void fill_stage(const std::vector<const FusedGate *> &gates, const std::vector<i
             if (!((used >> t) & 1)) free_bits.push_back(t);
         lane_bits(free_bits, &order);
         o.nb = (unsigned char)order.size();
-        for (size_t b = 0; b < order.size(); ++b) o.gv[b] = (unsigned short)addr_vec(order[b]);
-        o.moff = (unsigned short)(at / 4);
+        for (size_t b = 0; b < order.size(); ++b) {
+            const unsigned v = addr_vec(order[b]);
+            if (b < 10) o.lane[b % 5] |= b < 5 ? v : v << 16;
+            if (b >= 5) o.step[b - 5] = (unsigned short)v;
+        }
+        o.moff = (unsigned short)((image->size() - at0) / 4);
         const int D = 1 << g.k;
         for (int j = 0; j < D; ++j)
             for (int p = 0; p < D / 2; ++p) {
                 const size_t e0 = size_t(2 * p) * D + j, e1 = e0 + D;
-                mat[at++] = g.ur[e0];
-                mat[at++] = g.ur[e1];
-                mat[at++] = g.ui[e0];
-                mat[at++] = g.ui[e1];
+                image->push_back(g.ur[e0]);
+                image->push_back(g.ur[e1]);
+                image->push_back(g.ui[e0]);
+                image->push_back(g.ui[e1]);
             }
+        std::memcpy(image->data() + at0 + s * kGateFloats, &o, sizeof(o));
     }
+    a->units = (int)((image->size() - at0) / 4);
 }
 
 }  // namespace
@@ -246,13 +311,19 @@ void fill_stage(const std::vector<const FusedGate *> &gates, const std::vector<i
 void plan_passes(const std::vector<const FusedGate *> &gates, int n, PassPlan *plan)
 {
     plan->steps.clear();
+    plan->image.clear();
     std::vector<int> left;
-    bool reorder = true;
+    bool reorder = true, small = true;
     for (size_t i = 0; i < gates.size(); ++i) {
         left.push_back((int)i);
         if (gates[i]->path == SV_PATH_TC_TF32 || gates[i]->path == SV_PATH_TC_BF16X3) reorder = false;
+        if (gates[i]->k > 2) small = false;
     }
-    const int L = std::min(n, kStageQubits);
+    // Large tiles hold more gates a pass; on a small state they leave SMs without a tile, and a pass is
+    // then as long as its chain of gates on one tile.  Measured (us, tiles of 2^10 / 2^11 / 2^12):
+    // 16 qubits, gates of 2: 68 / 79 / 103, of 4: 86 / 65 / 67; 18 qubits, 2: 82 / 62 / 78;
+    // 19 qubits, 3: 139 / 94 / 72; 22 qubits, 4: 573 / 464 / 278.
+    const int L = std::min(n, n >= 19 ? kStageQubits : n <= 16 && small ? kStageQubits - 2 : kStageQubits - 1);
     while (!left.empty()) {
         PassStep st;
         uint64_t lam = 31, blocked = 0;
@@ -287,11 +358,11 @@ void plan_passes(const std::vector<const FusedGate *> &gates, int n, PassPlan *p
             st.single = took[0];
         } else {
             for (int q = 5; q < n && __builtin_popcountll(lam) < L; ++q) lam |= uint64_t(1) << q;   // whole tiles: lowest free qubits
-            st.form = mats <= size_t(kStageMat[0]) ? 0 : mats <= size_t(kStageMat[1]) ? 1 : 2;
+            for (int t : took) st.kmax = std::max(st.kmax, gates[(size_t)t]->k);
             st.tiles = 1ll << (n - L);
-            st.args.assign((sizeof(StageHead) + sizeof(float) * (size_t)kStageMat[st.form]) / 8, 0);
-            StageHead *h = reinterpret_cast<StageHead *>(st.args.data());
-            fill_stage(gates, took, lam, n, h, reinterpret_cast<float *>(h + 1));
+            st.image_off = plan->image.size();
+            st.args.assign((sizeof(StageArgs) + 7) / 8, 0);
+            fill_stage(gates, took, lam, n, reinterpret_cast<StageArgs *>(st.args.data()), &plan->image);
         }
         plan->steps.push_back(std::move(st));
         left.swap(rest);
@@ -300,37 +371,62 @@ void plan_passes(const std::vector<const FusedGate *> &gates, int n, PassPlan *p
 
 namespace {
 
-template <int T, int V, int M>
-int launch_form(float *sv, const PassStep &p, cudaStream_t stream)
+std::mutex g_stage_mu;
+uint64_t g_stage_attr[2][6] = {};   // by form and largest gate: a bit per device
+
+template <int T, int KMAX>
+int launch_form(float *sv, const float *image, const PassStep &p, cudaStream_t stream)
 {
-    static_assert(sizeof(StageArgs<M>) == sizeof(StageHead) + sizeof(float) * M, "a step's argument block is the kernel's");
-    const StageArgs<M> *a = reinterpret_cast<const StageArgs<M> *>(p.args.data());
-    const size_t smem = sizeof(float) * (size_t(64) << a->h.t.fb);
-    static_assert((8 << kStageQubits) <= 48 * 1024, "tiles need no shared-memory attribute");
-    void *args[2] = {&sv, const_cast<StageArgs<M> *>(a)};
-    SV_CUDA_TRY(cudaLaunchKernel(reinterpret_cast<const void *>(stage_kernel<T, V, M>), dim3((unsigned)p.tiles), dim3(T), args, smem, stream));
+    const StageArgs *a = reinterpret_cast<const StageArgs *>(p.args.data());
+    auto kern = stage_kernel<T, KMAX>;
+    int dev = 0;
+    SV_CUDA_TRY(cudaGetDevice(&dev));
+    const uint64_t bit = dev >= 0 && dev < 64 ? (1ull << dev) : 0ull;
+    {
+        uint64_t &slot = g_stage_attr[T == 512][KMAX];
+        std::lock_guard<std::mutex> lk(g_stage_mu);
+        if (!(slot & bit) || !bit) {
+            SV_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (8 << kStageQubits) + kStageMaxGates * (int)sizeof(StageGate) + 4 * kStageMatFloats));
+            slot |= bit;
+        }
+    }
+    // launched while the kernel before it drains (it waits for that one before it reads the state):
+    // 1.8 us from launch to launch instead of 3.1
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)p.tiles);
+    cfg.blockDim = dim3(T);
+    cfg.dynamicSmemBytes = (size_t(256) << a->t.fb) + 16 * (size_t)a->units;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    SV_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, sv, reinterpret_cast<const uint4 *>(image), *a));
     return SV_OK;
 }
 
-template <int M>
-int launch_mat(float *sv, const PassStep &p, cudaStream_t stream, int num_sms)
+template <int T>
+int launch_kmax(float *sv, const float *image, const PassStep &p, cudaStream_t stream)
 {
-    // With few tiles a pass is a chain of short gates, so each tile gets all the threads an SM
-    // takes; with many, small CTAs of two groups a thread share an SM and overlap each other's
-    // loads, barriers and arithmetic.
-    if (p.tiles < 2ll * num_sms) return launch_form<512, 1, M>(sv, p, stream);
-    return launch_form<128, 2, M>(sv, p, stream);
+    switch (p.kmax) {
+    case 1:
+    case 2: return launch_form<T, 2>(sv, image, p, stream);
+    case 3: return launch_form<T, 3>(sv, image, p, stream);
+    case 4: return launch_form<T, 4>(sv, image, p, stream);
+    default: return launch_form<T, 5>(sv, image, p, stream);
+    }
 }
 
 }  // namespace
 
-int launch_stage(float *sv, const PassStep &p, cudaStream_t stream, int num_sms)
+int launch_stage(float *sv, const float *image, const PassStep &p, cudaStream_t stream, int num_sms)
 {
-    switch (p.form) {
-    case 0: return launch_mat<kStageMat[0]>(sv, p, stream, num_sms);
-    case 1: return launch_mat<kStageMat[1]>(sv, p, stream, num_sms);
-    default: return launch_mat<kStageMat[2]>(sv, p, stream, num_sms);
-    }
+    // With few tiles a pass is a chain of short gates, so each tile gets all the threads an SM
+    // takes; with many, small CTAs of several groups a thread share an SM and overlap each other's
+    // loads, barriers and arithmetic.
+    return p.tiles < 2ll * num_sms ? launch_kmax<512>(sv, image + p.image_off, p, stream) : launch_kmax<128>(sv, image + p.image_off, p, stream);
 }
 
 }  // namespace svg

@@ -55,7 +55,7 @@ def bound(B, f):
     return sum((2 ** (B.sv_fused_get_info(f, i)["k"] + 1) + 2) * 2.0 ** -24 for i in range(B.sv_fused_count(f)))
 
 
-@pytest.mark.parametrize("n", [3, 5, 6, 9, 11, 12, 13, 14, 17, 20])
+@pytest.mark.parametrize("n", [3, 5, 6, 9, 11, 12, 13, 14, 17, 20, 22])
 @pytest.mark.parametrize("max_k", [1, 2, 3, 4, 5])
 def test_passes_match_oracle_and_single_launches(B, n, max_k):
     rng = np.random.default_rng(1000 * n + max_k)
