@@ -20,6 +20,7 @@
 // the shared-memory pipe: a thread therefore takes four groups at a time for k <= 3 and two for k = 4,
 // so that one such load serves 8 to 16 packed multiply-adds.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <mutex>
 
@@ -230,6 +231,7 @@ __global__ void __launch_bounds__(T, T == 128 ? stage_ctas(KMAX) : 1) stage_kern
 }
 
 // ------------------------------------------------------------------------------------ planner
+constexpr int kLargeQubits = 21;        // from 512 tiles on (the many-tile form)
 constexpr int kStageMatFloats = 4096;   // matrices of one pass: 16 KB, so that four CTAs share an SM
 
 bool stageable(const FusedGate &g)
@@ -237,6 +239,17 @@ bool stageable(const FusedGate &g)
     if (!g.post.empty() || !g.swaps.empty()) return false;
     if (g.path == SV_PATH_CONTROLLED) return g.k >= 1 && g.k <= 3;
     return (g.path == SV_PATH_LOW || g.path == SV_PATH_HIGH || g.path == SV_PATH_MIXED) && g.k >= 1 && g.k <= 5 && g.cmask == 0;
+}
+
+// Time of a gate on its own kernel, and its share in a pass, on states past the L2 in units of one read
+// and write of the state at the copy rate (k = 1..5; 28 qubits: 1.0 = 0.63 ms).  A pass adds
+// kPassCost for its own read and write, partly hidden behind the arithmetic.
+constexpr double kPassCost = 0.7, kInPass[6] = {0, 0.2, 0.3, 0.5, 1.0, 2.0};
+double alone_cost(const FusedGate &g)
+{
+    static const double high[6] = {0, 0.97, 0.97, 0.97, 1.09, 2.4}, tile[6] = {0, 0.97, 1.0, 1.2, 1.55, 4.0};
+    if (g.path == SV_PATH_CONTROLLED) return std::ldexp(1.0, -__builtin_popcountll(g.cmask & ~uint64_t(7)));
+    return g.path == SV_PATH_HIGH ? high[g.k] : tile[g.k];
 }
 
 uint64_t named(const FusedGate &g)
@@ -354,8 +367,24 @@ void plan_passes(const std::vector<const FusedGate *> &gates, int n, PassPlan *p
                 break;
             }
         }
-        if (took.size() == 1) {
-            st.single = took[0];
+        // On large states the one-gate kernels of four-qubit gates on high qubits run near the copy rate:
+        // a pass of two or three of those alone costs more than it saves.
+        bool pass = took.size() > 1;
+        if (pass && n >= kLargeQubits) {
+            double alone = 0, in = kPassCost;
+            for (int t : took) {
+                alone += alone_cost(*gates[(size_t)t]);
+                in += kInPass[gates[(size_t)t]->k];
+            }
+            pass = in < alone;
+        }
+        if (!pass) {
+            for (size_t t = 0; t + 1 < took.size(); ++t) {
+                PassStep one;
+                one.single = took[t];
+                plan->steps.push_back(std::move(one));
+            }
+            st.single = took.back();
         } else {
             for (int q = 5; q < n && __builtin_popcountll(lam) < L; ++q) lam |= uint64_t(1) << q;   // whole tiles: lowest free qubits
             for (int t : took) st.kmax = std::max(st.kmax, gates[(size_t)t]->k);
