@@ -153,132 +153,188 @@ __global__ void __launch_bounds__(kRedThreads) norm_kernel(const float *__restri
 }
 
 // ---------------------------------------------------------------------------------------------
-// sampling: chunk sums (fp64 via float-float per lane), exclusive prefix, then one warp per sample
-__global__ void chunk_sum_kernel(const float *__restrict__ sv, long long n_chunks, int chunk_blocks_log2,
-                                 double *__restrict__ chunk_sum)
+// sampling: chunk sums (float-float per thread, fp64 across threads), exclusive prefix, then one CTA
+// per sample.  One CTA sums a chunk of up to 2^14 amplitudes: a state of 2^20 has 64 chunks, which one
+// warp each left as 64 serial walks (n = 20, 1024 samples: 371 us for the whole call).
+constexpr int kChunkThreads = 256;
+
+__device__ __forceinline__ double ff_value(const FF &a) { return (double)a.hi + (double)a.lo; }
+
+// |re|^2 + |im|^2 of `items` 16-byte pairs (item i: block i >> 3, quarter i & 7) of the blocks at
+// `base`, taken first, first + step, ...: a chain each for the real and the imaginary parts
+__device__ __forceinline__ double sum_items(const float *__restrict__ base, int first, int step, int items)
 {
-    const int lane = threadIdx.x & 31;
-    long long w = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const long long stride = (long long)gridDim.x * (blockDim.x >> 5);
-    const long long cb = 1ll << chunk_blocks_log2;
-    for (; w < n_chunks; w += stride) {
-        FF acc{0.f, 0.f};
-        const float *base = sv + (w << chunk_blocks_log2) * 64;
-        for (long long b = 0; b < cb; ++b) {
-            ff_add_sq(acc, base[b * 64 + lane]);
-            ff_add_sq(acc, base[b * 64 + 32 + lane]);
-        }
-        double v = warp_sum_d((double)acc.hi + (double)acc.lo);
-        if (lane == 0) chunk_sum[w] = v;
+    FF re{0.f, 0.f}, im{0.f, 0.f};
+#pragma unroll 8
+    for (int i = first; i < items; i += step) {
+        const float *b = base + (i >> 3) * 64 + (i & 7) * 4;
+        const float4 r = *reinterpret_cast<const float4 *>(b);
+        const float4 m = *reinterpret_cast<const float4 *>(b + 32);
+        ff_add_sq(re, r.x); ff_add_sq(im, m.x);
+        ff_add_sq(re, r.y); ff_add_sq(im, m.y);
+        ff_add_sq(re, r.z); ff_add_sq(im, m.z);
+        ff_add_sq(re, r.w); ff_add_sq(im, m.w);
+    }
+    return ff_value(re) + ff_value(im);
+}
+
+__global__ void __launch_bounds__(kChunkThreads) chunk_sum_kernel(const float *__restrict__ sv, int chunk_blocks_log2,
+                                                                  double *__restrict__ chunk_sum)
+{
+    __shared__ double ws[kChunkThreads / 32];
+    const double v = warp_sum_d(sum_items(sv + ((long long)blockIdx.x << chunk_blocks_log2) * 64, (int)threadIdx.x, kChunkThreads,
+                                          8 << chunk_blocks_log2));
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double s = 0.0;
+#pragma unroll
+        for (int i = 0; i < kChunkThreads / 32; ++i) s += ws[i];
+        chunk_sum[blockIdx.x] = s;
     }
 }
 
-// single CTA exclusive scan of n chunk sums (in: sums, out: prefix), total at prefix[n]
+// inclusive warp scan
+__device__ __forceinline__ double warp_scan_d(double v, int lane)
+{
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const double t = __shfl_up_sync(0xffffffffu, v, d);
+        if (lane >= d) v += t;
+    }
+    return v;
+}
+
+// single CTA exclusive scan of n chunk sums (in: sums, out: prefix), total at prefix[n]:
+// each thread sums its own range, the 1024 range sums are scanned by warps, then each thread writes
+// its range
 __global__ void __launch_bounds__(1024) chunk_scan_kernel(const double *__restrict__ sums, double *__restrict__ prefix, long long n)
 {
-    __shared__ double seg[1024];
+    __shared__ double seg[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long per = (n + 1023) / 1024;
-    const long long lo = threadIdx.x * per;
+    const long long lo = threadIdx.x * per < n ? threadIdx.x * per : n;
     const long long hi = lo + per < n ? lo + per : n;
     double s = 0.0;
+#pragma unroll 8
     for (long long i = lo; i < hi; ++i) s += sums[i];
-    seg[threadIdx.x] = s;
+    const double incl = warp_scan_d(s, lane);
+    if (lane == 31) seg[warp] = incl;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double run = 0.0;
-        for (int t = 0; t < 1024; ++t) {
-            double v = seg[t];
-            seg[t] = run;
-            run += v;
+    if (warp == 0) {
+        const double t = warp_scan_d(seg[lane], lane);
+        __syncwarp();
+        seg[lane] = t;
+        if (lane == 31) {
+            prefix[n] = t;
         }
-        prefix[n] = run;
     }
     __syncthreads();
-    double run = seg[threadIdx.x];
+    double run = (incl - s) + (warp ? seg[warp - 1] : 0.0);
+#pragma unroll 8
     for (long long i = lo; i < hi; ++i) {
         prefix[i] = run;
         run += sums[i];
     }
 }
 
-// One CTA of kSearchWarps warps per sample; p_i = re^2 + im^2 in fp64 (products of widened
-// floats are exact).  After the chunk holding the sample is found (binary search on the chunk
-// prefix sums), each warp sums p over its own part of the chunk with independent loads; thread 0
-// picks the part where the running total passes the target; one warp then walks that part 32
-// amplitudes at a time (warp scan) to the first index whose running total exceeds it, going on
-// into the next part if the walk's rounding leaves the target just past this part's end.
-constexpr int kSearchWarps = 8;
+// One CTA per sample; p_i = re^2 + im^2 in fp64 (products of widened floats are exact).  The chunk
+// holding the sample is found by 256 probes of the chunk prefix sums at a time; each warp sums an
+// eighth of a full chunk (float-float: fp64 multiply-adds run at 2 a clock on an SM, and 16 K of them
+// a sample were the call's longest part); the eighth where the running total passes the target is
+// then walked 2048 amplitudes at a step, eight to a thread, with a scan over the CTA, to the first
+// index whose running total exceeds it, going on past the eighth if rounding leaves the target
+// just past its end.
+constexpr int kSearchThreads = 256;
+constexpr int kSearchStep = 8 * kSearchThreads;
 
-__global__ void __launch_bounds__(32 * kSearchWarps) sample_search_kernel(const float *__restrict__ sv, int n, long long n_chunks,
-                                                                          int chunk_log2, const double *__restrict__ prefix,
-                                                                          const double *__restrict__ uniforms, int n_samples,
-                                                                          unsigned long long *__restrict__ out)
+__global__ void __launch_bounds__(kSearchThreads) sample_search_kernel(const float *__restrict__ sv, int n, long long n_chunks,
+                                                                       int chunk_log2, const double *__restrict__ prefix,
+                                                                       const double *__restrict__ uniforms, int n_samples,
+                                                                       unsigned long long *__restrict__ out)
 {
-    __shared__ double part[kSearchWarps];
-    __shared__ int s_part;
-    __shared__ double s_run;
+    __shared__ double part[kSearchThreads / 32];
+    __shared__ int s_first;
     const int s = blockIdx.x;
     if (s >= n_samples) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const double total = prefix[n_chunks];
-    const double target = uniforms[s] * total;
-    // largest chunk c with prefix[c] <= target
-    long long lo = 0, hi = n_chunks - 1;
-    while (lo < hi) {
-        long long mid = (lo + hi + 1) >> 1;
-        if (prefix[mid] <= target) lo = mid; else hi = mid - 1;
+    const double target = uniforms[s] * prefix[n_chunks];
+    // largest chunk c with prefix[c] <= target, in [lo, lo + len)
+    long long lo = 0, len = n_chunks;
+    while (len > 1) {
+        const long long step = (len + kSearchThreads - 1) / kSearchThreads;
+        const long long off = (long long)threadIdx.x * step;
+        const int below = __syncthreads_count(off < len && prefix[lo + off] <= target);
+        const long long at = below > 0 ? (long long)(below - 1) * step : 0;
+        lo += at;
+        len = step < len - at ? step : len - at;
     }
     const unsigned long long N = 1ull << n;
-    const unsigned long long i0 = (unsigned long long)lo << chunk_log2;
-    const unsigned long long part_amps = (1ull << chunk_log2) / kSearchWarps;
-    double acc = 0.0;
-    for (unsigned long long k = lane; k < part_amps; k += 32) {
-        const unsigned long long i = i0 + (unsigned long long)warp * part_amps + k;
-        if (i < N) {
-            const long long o = re_off(i);
-            const double re = (double)sv[o], im = (double)sv[o + 32];
-            acc += re * re + im * im;
-        }
+    unsigned long long i0 = (unsigned long long)lo << chunk_log2;
+    double run = prefix[lo];
+    if (chunk_log2 == kChunkLog2) {
+        constexpr int kItems = (1 << kChunkLog2) / 4 / (kSearchThreads / 32);   // a warp's 16-byte pairs
+        const double v = warp_sum_d(sum_items(sv + (long long)(i0 >> 5) * 64 + (long long)warp * kItems * 8, lane, 32, kItems));
+        if (lane == 0) part[warp] = v;
+        __syncthreads();
+        int p = 0;   // every thread: the same sums in the same order
+        while (p < kSearchThreads / 32 - 1 && run + part[p] <= target) run += part[p++];
+        i0 += (unsigned long long)p * ((1u << kChunkLog2) / (kSearchThreads / 32));
+        __syncthreads();
     }
+    for (;; i0 += kSearchStep) {
+        // thread t: amplitudes i0 + 8 t .. + 7
+        const unsigned long long i = i0 + 8ull * threadIdx.x;
+        double p[8];
+        double own = 0.0;
+        const bool in = i < N;   // N < 8 (n < 3): the block is zero-padded, and the answer is clamped
+        if (in) {
+            const float *b = sv + re_off(i);
+            const float4 r0 = *reinterpret_cast<const float4 *>(b), r1 = *reinterpret_cast<const float4 *>(b + 4);
+            const float4 m0 = *reinterpret_cast<const float4 *>(b + 32), m1 = *reinterpret_cast<const float4 *>(b + 36);
+            const float re[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
+            const float im[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
-    if (lane == 0) part[warp] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double run = prefix[lo];
-        int p = 0;
-        while (p < kSearchWarps - 1 && run + part[p] <= target) run += part[p++];
-        s_part = p;
-        s_run = run;
-    }
-    __syncthreads();
-    if (warp != 0) return;
-    double run = s_run;
-    unsigned long long answer = N - 1;
-    bool found = false;
-    for (unsigned long long base = i0 + (unsigned long long)s_part * part_amps; base < N && !found; base += 32) {
-        const unsigned long long i = base + lane;
-        double p = 0.0;
-        if (i < N) {
-            const long long o = re_off(i);
-            const double re = (double)sv[o], im = (double)sv[o + 32];
-            p = re * re + im * im;
+            for (int e = 0; e < 8; ++e) {
+                p[e] = (double)re[e] * (double)re[e] + (double)im[e] * (double)im[e];
+                own += p[e];
+            }
         }
-        // inclusive warp scan
-        double incl = p;
+        const double incl = warp_scan_d(own, lane);
+        if (lane == 31) part[warp] = incl;
+        if (threadIdx.x == 0) s_first = kSearchThreads;
+        __syncthreads();
+        double before = run;
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            double t = __shfl_up_sync(0xffffffffu, incl, d);
-            if (lane >= d) incl += t;
+        for (int w = 0; w < kSearchThreads / 32; ++w) {
+            if (w < warp) before += part[w];
+            run += part[w];
         }
-        const unsigned hit = __ballot_sync(0xffffffffu, (i < N) && (run + incl > target));
-        if (hit) {
-            answer = base + (unsigned long long)(__ffs(hit) - 1);
-            found = true;
+        const bool hit = in && before + incl > target;
+        if (hit) atomicMin(&s_first, (int)threadIdx.x);
+        __syncthreads();
+        const int first = s_first;
+        if (first < kSearchThreads) {
+            if ((int)threadIdx.x == first) {
+                double t = before + (incl - own);
+                int e = 0;
+#pragma unroll
+                for (int q = 0; q < 7; ++q)
+                    if (e == q) {
+                        t += p[q];
+                        if (!(t > target)) e = q + 1;
+                    }
+                const unsigned long long a = i + (unsigned)e;
+                out[s] = a < N ? a : N - 1;
+            }
+            return;
         }
-        run += __shfl_sync(0xffffffffu, incl, 31);
+        if (i0 + kSearchStep >= N) {
+            if (threadIdx.x == 0) out[s] = N - 1;
+            return;
+        }
+        __syncthreads();   // part and s_first are written again
     }
-    if (lane == 0) out[s] = answer;
 }
 
 int grid_for(long long items, int threads, int num_sms, int per_sm)
@@ -490,12 +546,12 @@ int sample_impl(sv_state *st, const double *uniforms, int n_samples, uint64_t *o
     if (st->c128) {
         SV_TRY(c128_sample(st, n_samples));
     } else {
-        chunk_sum_kernel<<<grid_for(nc * 32, 256, st->num_sms, 8), 256, 0, st->stream>>>(st->d, nc, chunk_blocks_log2, sums);
+        chunk_sum_kernel<<<(unsigned)nc, kChunkThreads, 0, st->stream>>>(st->d, chunk_blocks_log2, sums);
         SV_CUDA_TRY(cudaGetLastError());
         chunk_scan_kernel<<<1, 1024, 0, st->stream>>>(sums, prefix, nc);
         SV_CUDA_TRY(cudaGetLastError());
         if (n_samples > 0) {
-            sample_search_kernel<<<n_samples, 32 * kSearchWarps, 0, st->stream>>>(st->d, n, nc, chunk_log2, prefix, st->d_uniforms,
+            sample_search_kernel<<<n_samples, kSearchThreads, 0, st->stream>>>(st->d, n, nc, chunk_log2, prefix, st->d_uniforms,
                                                                                  n_samples, st->d_samples);
             SV_CUDA_TRY(cudaGetLastError());
         }
@@ -582,7 +638,6 @@ extern "C" int sv_sample_noalloc(const void *dev_state, int n_qubits, void *cuda
     double *scratch = nullptr;
     SV_TRY(noalloc_scratch(device, &scratch));
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    const int num_sms = device_sm_count(device);
     const int n = n_qubits;
     const int chunk_log2 = n > kChunkLog2 ? kChunkLog2 : (n >= 5 ? n : 5);
     const long long nc = n > kChunkLog2 ? (1ll << (n - kChunkLog2)) : 1ll;
@@ -592,11 +647,11 @@ extern "C" int sv_sample_noalloc(const void *dev_state, int n_qubits, void *cuda
     unsigned long long *d_out = reinterpret_cast<unsigned long long *>(d_u + kNoAllocMaxSamples);
     const float *sv = static_cast<const float *>(dev_state);
     SV_CUDA_TRY(cudaMemcpyAsync(d_u, uniforms, sizeof(double) * size_t(n_samples), cudaMemcpyHostToDevice, stream));
-    chunk_sum_kernel<<<grid_for(nc * 32, 256, num_sms, 8), 256, 0, stream>>>(sv, nc, chunk_log2 - 5, sums);
+    chunk_sum_kernel<<<(unsigned)nc, kChunkThreads, 0, stream>>>(sv, chunk_log2 - 5, sums);
     SV_CUDA_TRY(cudaGetLastError());
     chunk_scan_kernel<<<1, 1024, 0, stream>>>(sums, prefix, nc);
     SV_CUDA_TRY(cudaGetLastError());
-    sample_search_kernel<<<n_samples, 32 * kSearchWarps, 0, stream>>>(sv, n, nc, chunk_log2, prefix, d_u, n_samples, d_out);
+    sample_search_kernel<<<n_samples, kSearchThreads, 0, stream>>>(sv, n, nc, chunk_log2, prefix, d_u, n_samples, d_out);
     SV_CUDA_TRY(cudaGetLastError());
     SV_CUDA_TRY(cudaMemcpyAsync(out, d_out, sizeof(unsigned long long) * size_t(n_samples), cudaMemcpyDeviceToHost, stream));
     SV_CUDA_TRY(cudaStreamSynchronize(stream));
