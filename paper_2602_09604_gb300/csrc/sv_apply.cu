@@ -25,6 +25,7 @@
 #include <mutex>
 
 #include "sv_internal.h"
+#include "sv_launch.h"
 
 namespace svg {
 namespace {
@@ -181,10 +182,12 @@ __global__ void __launch_bounds__(kHighThreads, high_min_blocks<K>()) apply_high
     constexpr int TPB = 32 / V;
     constexpr int D = 1 << K;
     extern __shared__ float2 s_u[];
+    next_may_start();
     if constexpr (K == 6) {
         for (int i = threadIdx.x; i < D * D; i += blockDim.x) s_u[i] = umem[i];
         __syncthreads();
     }
+    wait_for_previous();
     const long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (w >= a.n_items) return;
     unsigned long long blk = (unsigned long long)w / TPB;
@@ -252,6 +255,7 @@ __global__ void __launch_bounds__(kTileThreads, tile_min_blocks<K>()) apply_tile
 {
     constexpr int D = 1 << K;
     extern __shared__ __align__(16) float smem[];
+    next_may_start();
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int f = FIXED ? tile_f<K>() : a.t.f;
@@ -262,6 +266,7 @@ __global__ void __launch_bounds__(kTileThreads, tile_min_blocks<K>()) apply_tile
         for (int i = threadIdx.x; i < D * D; i += blockDim.x) s_u[i] = umem[i];
         __syncthreads();
     }
+    wait_for_previous();
     const long long t = (long long)blockIdx.x * kTileWarps + warp;
     if (t >= a.t.n_tiles) return;
     unsigned long long b0 = (unsigned long long)t;
@@ -414,6 +419,8 @@ template <int K>
 __global__ void __launch_bounds__(kHighThreads) apply_ctrl_kernel(float *__restrict__ sv, const __grid_constant__ CtrlArgs<K> a)
 {
     constexpr int D = 1 << K;
+    next_may_start();
+    wait_for_previous();
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= a.n_groups) return;
     unsigned long long b = (unsigned long long)g;
@@ -460,9 +467,7 @@ int launch_ctrl(float *sv, int n, const FusedGate &g, const float2 *, cudaStream
     a.cmask = g.cmask;
     a.n_groups = 1ll << (n - np);
     const long long grid = (a.n_groups + kHighThreads - 1) / kHighThreads;
-    apply_ctrl_kernel<K><<<(unsigned)grid, kHighThreads, 0, stream>>>(sv, a);
-    SV_CUDA_TRY(cudaGetLastError());
-    return SV_OK;
+    return launch_chained(true, apply_ctrl_kernel<K>, (unsigned)grid, kHighThreads, 0, stream, sv, a);
 }
 
 template <int K>
@@ -492,9 +497,7 @@ int launch_high(float *sv, int n, const FusedGate &g, const float2 *umem, cudaSt
     }
     (void)num_sms;
     const long long grid = (a.n_items + kHighThreads - 1) / kHighThreads;
-    kern<<<(unsigned)grid, kHighThreads, smem, stream>>>(sv, a, umem);
-    SV_CUDA_TRY(cudaGetLastError());
-    return SV_OK;
+    return launch_chained(true, kern, (unsigned)grid, kHighThreads, smem, stream, sv, a, umem);
 }
 
 template <int K>
@@ -524,9 +527,7 @@ int launch_tile(float *sv, int n, const FusedGate &g, const float2 *umem, cudaSt
     }
     (void)num_sms;
     const long long grid = (a.t.n_tiles + kTileWarps - 1) / kTileWarps;
-    kern<<<(unsigned)grid, kTileThreads, smem, stream>>>(sv, a, umem);
-    SV_CUDA_TRY(cudaGetLastError());
-    return SV_OK;
+    return launch_chained(true, kern, (unsigned)grid, kTileThreads, smem, stream, sv, a, umem);
 }
 
 using LaunchFn = int (*)(float *, int, const FusedGate &, const float2 *, cudaStream_t, int);

@@ -25,6 +25,7 @@
 #include <mutex>
 
 #include "sv_internal.h"
+#include "sv_launch.h"
 #include "sv_tile.h"
 
 namespace svg {
@@ -195,15 +196,14 @@ __global__ void __launch_bounds__(T, T == 128 ? stage_ctas(KMAX) : 1) stage_kern
                                                                                  const __grid_constant__ StageArgs a)
 {
     extern __shared__ __align__(16) float tile[];
-    // The pass after this one may start its own set-up; the state is read once the one before is done.
-    asm volatile("griddepcontrol.launch_dependents;");
+    next_may_start();
     uint4 *img = reinterpret_cast<uint4 *>(tile + (64 << a.t.fb));
     for (int i = threadIdx.x; i < a.units; i += T) img[i] = __ldg(image + i);
     const TileMover<T> mv(a.t);
     const ThreadMasks tm;
     const unsigned long long b0 = tile_base(a.t, blockIdx.x);
     float *g0 = sv + (long long)(b0 << 6);
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    wait_for_previous();
     mv.load(a.t, g0, tile);
     __syncthreads();
     constexpr bool F = T == 512;   // few tiles: one group at a time, so that more threads have one
@@ -420,20 +420,8 @@ int launch_form(float *sv, const float *image, const PassStep &p, cudaStream_t s
             slot |= bit;
         }
     }
-    // launched while the kernel before it drains (it waits for that one before it reads the state):
-    // 1.8 us from launch to launch instead of 3.1
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)p.tiles);
-    cfg.blockDim = dim3(T);
-    cfg.dynamicSmemBytes = (size_t(256) << a->t.fb) + 16 * (size_t)a->units;
-    cfg.stream = stream;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    SV_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, sv, reinterpret_cast<const uint4 *>(image), *a));
-    return SV_OK;
+    return launch_chained(true, kern, (unsigned)p.tiles, T, (size_t(256) << a->t.fb) + 16 * (size_t)a->units, stream, sv,
+                          reinterpret_cast<const uint4 *>(image), *a);
 }
 
 template <int T>

@@ -36,6 +36,7 @@
 #include <type_traits>
 
 #include "sv_internal.h"
+#include "sv_launch.h"
 
 namespace svg {
 namespace {
@@ -280,7 +281,8 @@ __device__ __forceinline__ float4 xor_perm4(float4 v, unsigned sw)
 //   4. one thread per warpgroup issues the MMAs (A from tensor memory, B from shared memory).
 // VS (direct variant only): inputs from the virtual source v instead of sv.  The body is inlined
 // into two entry points so the kernels without a virtual source keep their own parameter block.
-template <int K, int MODE, bool STAGED, bool VS>
+// CH: launched behind the kernel before (sv_launch.h): the B image is read before the wait for it.
+template <int K, int MODE, bool STAGED, bool VS, bool CH>
 __device__ __forceinline__ void tc_kernel_body(float *__restrict__ sv, const TcArgs &a, const VsArgs &v)
 {
     using S = TcShape<K, MODE>;
@@ -297,6 +299,14 @@ __device__ __forceinline__ void tc_kernel_body(float *__restrict__ sv, const TcA
     volatile int *status = reinterpret_cast<volatile int *>(tslot + 1);   // [0], [1]: per warpgroup
     const uint32_t bar_b = smem_u32(&bars[0]);
     const uint32_t bar_mma = smem_u32(&bars[1 + wg]);
+    if constexpr (CH) next_may_start();
+    auto copy_b = [&]() {   // B image (written by no kernel): bulk copies of up to 32 KB, all completing on bar_b
+        mbar_arrive_expect_tx(bar_b, a.bbytes);
+        for (unsigned off = 0; off < a.bbytes; off += 32768u) {
+            const unsigned sz = a.bbytes - off < 32768u ? a.bbytes - off : 32768u;
+            bulk_g2s(smem_u32(sB + off), static_cast<const unsigned char *>(a.bimg) + off, sz, bar_b);
+        }
+    };
 
     if (tid == 0) {
         mbar_init(bar_b, 1);
@@ -306,7 +316,9 @@ __device__ __forceinline__ void tc_kernel_body(float *__restrict__ sv, const TcA
         status[1] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
+        if constexpr (CH) copy_b();
     }
+    if constexpr (CH) wait_for_previous();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
                      "r"((uint32_t)S::TMEM_COLS)
@@ -322,13 +334,7 @@ __device__ __forceinline__ void tc_kernel_body(float *__restrict__ sv, const TcA
     const uint32_t tA = t_wg;                                         // A image(s)
     const uint32_t tD = t_wg + (uint32_t)(S::NIMG * S::A_COLS);      // accumulator
 
-    if (tid == 0) {   // B image: bulk copies of up to 32 KB, all completing on bar_b
-        mbar_arrive_expect_tx(bar_b, a.bbytes);
-        for (unsigned off = 0; off < a.bbytes; off += 32768u) {
-            const unsigned sz = a.bbytes - off < 32768u ? a.bbytes - off : 32768u;
-            bulk_g2s(smem_u32(sB + off), static_cast<const unsigned char *>(a.bimg) + off, sz, bar_b);
-        }
-    }
+    if (!CH && tid == 0) copy_b();
 
     const uint32_t idesc = (1u << 4) | ((MODE == kModeTF32 ? 2u : 1u) << 7) | ((MODE == kModeTF32 ? 2u : 1u) << 10) |
                            ((uint32_t)(S::KD >> 3) << 17) | ((uint32_t)(kTcM >> 4) << 24);
@@ -596,18 +602,18 @@ __device__ __forceinline__ void tc_kernel_body(float *__restrict__ sv, const TcA
     }
 }
 
-template <int K, int MODE, bool STAGED>
+template <int K, int MODE, bool STAGED, bool CH>
 __global__ void __launch_bounds__(2 * kTcThreads, STAGED ? TcShape<K, MODE>::MIN_BLOCKS_STAGED : TcShape<K, MODE>::MIN_BLOCKS_DIRECT)
     apply_tc_kernel(float *__restrict__ sv, const __grid_constant__ TcArgs a)
 {
-    tc_kernel_body<K, MODE, STAGED, false>(sv, a, VsArgs{});
+    tc_kernel_body<K, MODE, STAGED, false, CH>(sv, a, VsArgs{});
 }
 
 template <int K, int MODE>
 __global__ void __launch_bounds__(2 * kTcThreads, TcShape<K, MODE>::MIN_BLOCKS_DIRECT)
     apply_tc_kernel_vs(float *__restrict__ sv, const __grid_constant__ TcArgs a, const __grid_constant__ VsArgs v)
 {
-    tc_kernel_body<K, MODE, false, true>(sv, a, v);
+    tc_kernel_body<K, MODE, false, true, false>(sv, a, v);
 }
 
 // ------------------------------------------------------------------------ warp-specialised kernel
@@ -686,7 +692,8 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-template <int MODE, bool VS, int LW, int EW, int WIN, bool V4, bool PH = false>
+// CH: launched behind the kernel before (sv_launch.h): the B image is read before the wait for it.
+template <int MODE, bool VS, int LW, int EW, int WIN, bool V4, bool CH, bool PH = false>
 __device__ __forceinline__ void tc_ws_body(float *__restrict__ sv, const TcArgs &a, const VsArgs &v)
 {
     using S = TcShape<6, MODE>;
@@ -708,6 +715,16 @@ __device__ __forceinline__ void tc_ws_body(float *__restrict__ sv, const TcArgs 
     const uint32_t bar_drain = smem_u32(&bars[W::N_BAR - 1]);
     const uint32_t sA0 = smem_u32(smem + W::OFF_A);
 
+    if constexpr (CH) next_may_start();
+    // bulk copies of up to 32 KB, all completing on bar_b
+    auto copy_b = [&]() {
+        const uint32_t b0 = smem_u32(smem);
+        mbar_arrive_expect_tx(bar_b, a.bbytes);
+        for (unsigned off = 0; off < a.bbytes; off += 32768u) {
+            const unsigned sz = a.bbytes - off < 32768u ? a.bbytes - off : 32768u;
+            bulk_g2s(b0 + off, static_cast<const unsigned char *>(a.bimg) + off, sz, bar_b);
+        }
+    };
     if (threadIdx.x == 0) {
         mbar_init(bar_b, 1);
         for (int s = 0; s < kWsStages; ++s) {
@@ -722,7 +739,9 @@ __device__ __forceinline__ void tc_ws_body(float *__restrict__ sv, const TcArgs 
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
+        if (CH && (long long)blockIdx.x < a.n_mma_tiles) copy_b();   // (written by no kernel)
     }
+    if constexpr (CH) wait_for_previous();
     if (warp == MMA_WARP) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
                      "r"((uint32_t)W::TMEM_COLS)
@@ -977,12 +996,8 @@ __device__ __forceinline__ void tc_ws_body(float *__restrict__ sv, const TcArgs 
                                ((uint32_t)(S::KD >> 3) << 17) | ((uint32_t)(kTcM >> 4) << 24);
         const uint32_t b0 = smem_u32(smem);
         bool b_done = false;
-        if (cnt > 0) {   // B image: bulk copies of up to 32 KB, all completing on bar_b
-            mbar_arrive_expect_tx(bar_b, a.bbytes);
-            for (unsigned off = 0; off < a.bbytes; off += 32768u) {
-                const unsigned sz = a.bbytes - off < 32768u ? a.bbytes - off : 32768u;
-                bulk_g2s(b0 + off, static_cast<const unsigned char *>(a.bimg) + off, sz, bar_b);
-            }
+        if (cnt > 0) {
+            if constexpr (!CH) copy_b();
             b_done = wait(bar_b, 0, 0x10);
         }
         for (long long i = 0; b_done && i < cnt; ++i) {
@@ -1033,17 +1048,17 @@ constexpr int kWsThreads = (kWsLoadWarps + kWsEpiWarps + 1) * 32;
 
 // V4: the gate's two lowest targets are qubits 0 and 1, so the loaders move four members of a group
 // with one 16-byte access (a warp's accesses are then whole lines)
-template <int MODE, bool V4>
+template <int MODE, bool V4, bool CH>
 __global__ void __launch_bounds__(kWsThreads, 1) apply_tc_ws_kernel(float *__restrict__ sv, const __grid_constant__ TcArgs a)
 {
-    tc_ws_body<MODE, false, kWsLoadWarps, kWsEpiWarps, kWsWindow, V4>(sv, a, VsArgs{});
+    tc_ws_body<MODE, false, kWsLoadWarps, kWsEpiWarps, kWsWindow, V4, CH>(sv, a, VsArgs{});
 }
 
 template <int MODE>
 __global__ void __launch_bounds__(kWsThreads, 1)
     apply_tc_ws_kernel_vs(float *__restrict__ sv, const __grid_constant__ TcArgs a, const __grid_constant__ VsArgs v)
 {
-    tc_ws_body<MODE, true, kWsLoadWarps, kWsEpiWarps, kWsWindow, false>(sv, a, v);
+    tc_ws_body<MODE, true, kWsLoadWarps, kWsEpiWarps, kWsWindow, false, false>(sv, a, v);
 }
 
 // k = 6, at most two targets below qubit 5 (not both 0 and 1), with post-phases in the epilogue:
@@ -1051,10 +1066,10 @@ __global__ void __launch_bounds__(kWsThreads, 1)
 // at 72 registers, gave the loaders fewer registers and ran 2% slower)
 constexpr int kWsPhEpiWarps = 4;
 constexpr int kWsPhThreads = (kWsLoadWarps + kWsPhEpiWarps + 1) * 32;
-template <int MODE>
+template <int MODE, bool CH>
 __global__ void __launch_bounds__(kWsPhThreads, 1) apply_tc_ws_kernel_ph(float *__restrict__ sv, const __grid_constant__ TcArgs a)
 {
-    tc_ws_body<MODE, false, kWsLoadWarps, kWsPhEpiWarps, kWsWindow, false, true>(sv, a, VsArgs{});
+    tc_ws_body<MODE, false, kWsLoadWarps, kWsPhEpiWarps, kWsWindow, false, CH, true>(sv, a, VsArgs{});
 }
 
 // ---------------------------------------------------------------------------------------- host
@@ -1225,9 +1240,14 @@ int launch_tc_t(float *sv, int n, const FusedGate &g, const void *dtc, cudaStrea
         a.ph = reinterpret_cast<const float *>(static_cast<const unsigned char *>(dtc) + ph_table_offset(K, MODE));
         a.ph_nb = (n + 7) / 8;
     }
+    // Past 2^26 amplitudes a pass takes 160 us and more and there is no launch gap left to win: those
+    // run the plain forms (chained, the staged k = 6 kernel took 3.89 ms instead of 3.69 at 30 qubits).
+    const bool chained = n <= 26 && !vs;
     VsArgs v{};
     if (vs) v = VsArgs{vs->src, vs->mask, vs->rest, vs->off};
-    void (*kern)(float *, const TcArgs) = staged ? apply_tc_kernel<K, MODE, true> : apply_tc_kernel<K, MODE, false>;
+    void (*kern)(float *, const TcArgs) =
+        chained ? (staged ? apply_tc_kernel<K, MODE, true, true> : apply_tc_kernel<K, MODE, false, true>)
+                : (staged ? apply_tc_kernel<K, MODE, true, false> : apply_tc_kernel<K, MODE, false, false>);
     void (*kern_vs)(float *, const TcArgs, const VsArgs) = apply_tc_kernel_vs<K, MODE>;
     int smem = staged ? S::SMEM_STAGED : S::SMEM_DIRECT;
     int tmem_cols = S::TMEM_COLS;
@@ -1236,7 +1256,8 @@ int launch_tc_t(float *sv, int n, const FusedGate &g, const void *dtc, cudaStrea
     if constexpr (K == 6) {   // the warp-specialised kernel exists for k = 6 only
         if (variant == 2) {
             const bool v4 = g.targets[0] == 0 && g.targets[1] == 1;
-            kern = ph ? apply_tc_ws_kernel_ph<MODE> : v4 ? apply_tc_ws_kernel<MODE, true> : apply_tc_ws_kernel<MODE, false>;
+            if (chained) kern = ph ? apply_tc_ws_kernel_ph<MODE, true> : v4 ? apply_tc_ws_kernel<MODE, true, true> : apply_tc_ws_kernel<MODE, false, true>;
+            else kern = ph ? apply_tc_ws_kernel_ph<MODE, false> : v4 ? apply_tc_ws_kernel<MODE, true, false> : apply_tc_ws_kernel<MODE, false, false>;
             kern_vs = apply_tc_ws_kernel_vs<MODE>;
             smem = WsShape<MODE>::SMEM;
             tmem_cols = WsShape<MODE>::TMEM_COLS;
@@ -1244,9 +1265,9 @@ int launch_tc_t(float *sv, int n, const FusedGate &g, const void *dtc, cudaStrea
             per_sm_regs = 1;
         }
     }
-    // function-attribute slot: variant, virtual source, 16-byte loaders, post-phases
-    const int akey = ph ? 9 : variant + (vs ? 3 : 0) + (variant == 2 && !vs && g.targets[0] == 0 && g.targets[1] == 1 ? 6 : 0);
-    static uint64_t attr_set[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};   // per kernel form, a bit per device (attributes are per device)
+    // function-attribute slot: chained, variant, virtual source, 16-byte loaders, post-phases
+    const int akey = (chained ? 10 : 0) + (ph ? 9 : variant + (vs ? 3 : 0) + (variant == 2 && !vs && g.targets[0] == 0 && g.targets[1] == 1 ? 6 : 0));
+    static uint64_t attr_set[20] = {};   // per kernel form, a bit per device (attributes are per device)
     {
         int dev = 0;
         SV_CUDA_TRY(cudaGetDevice(&dev));
@@ -1265,10 +1286,8 @@ int launch_tc_t(float *sv, int n, const FusedGate &g, const void *dtc, cudaStrea
     // the two-warpgroup kernels take two MMA tiles per CTA round, the warp-specialised one one
     const long long tiles_per_cta = variant == 2 ? 1 : 2;
     const long long grid = std::min<long long>((a.n_mma_tiles + tiles_per_cta - 1) / tiles_per_cta, (long long)num_sms * per_sm);
-    if (vs) kern_vs<<<(unsigned)grid, threads, smem, stream>>>(sv, a, v);
-    else kern<<<(unsigned)grid, threads, smem, stream>>>(sv, a);
-    SV_CUDA_TRY(cudaGetLastError());
-    return SV_OK;
+    if (vs) return launch_chained(false, kern_vs, (unsigned)grid, (unsigned)threads, (size_t)smem, stream, sv, a, v);
+    return launch_chained(chained, kern, (unsigned)grid, (unsigned)threads, (size_t)smem, stream, sv, a);
 }
 
 }  // namespace
