@@ -289,6 +289,7 @@ int launch_ev(const float *sv, const EvArgs &a, double *partials, unsigned *coun
 // name any qubit.  Terms of a pair (j, j ^ x) are equal once signed, so only one of each pair is formed.
 constexpr int kEvtThreads = 128;
 constexpr int kEvtQubits = 12;
+constexpr int kEvtCtas = 4;      // per SM: 53 KB of shared memory, 128 registers a thread
 constexpr int kEvtGroups = 32;
 constexpr int kEvtStrings = 64;
 
@@ -313,17 +314,16 @@ struct EvtArgs {
 
 __device__ __forceinline__ float pick_sign(float v, unsigned odd) { return __uint_as_float(__float_as_uint(v) ^ (odd << 31)); }
 
-__global__ void __launch_bounds__(kEvtThreads, 3) expval_tile_kernel(const float *__restrict__ sv, const __grid_constant__ EvtArgs a,
+__global__ void __launch_bounds__(kEvtThreads, kEvtCtas) expval_tile_kernel(const float *__restrict__ sv, const __grid_constant__ EvtArgs a,
                                                                      double *__restrict__ partials)
 {
     extern __shared__ __align__(16) float smem[];
     float *tile = smem;
-    float *red = smem + (64 << a.t.fb);                                   // two buffers of 16 x 128 entries
-    float2 *acc = reinterpret_cast<float2 *>(red + 2 * 16 * kEvtThreads);   // per string and lane
+    float *rb = smem + (64 << a.t.fb);                              // 16 x 128 entries
+    float2 *acc = reinterpret_cast<float2 *>(rb + 16 * kEvtThreads);   // per string and lane
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const TileMover<kEvtThreads> mv(a.t);
     for (int i = tid; i < a.n_strings * 32; i += kEvtThreads) acc[i] = make_float2(0.f, 0.f);
-    int pb = 0;
     for (long long t = blockIdx.x; t < a.tiles; t += gridDim.x) {
         const unsigned long long b0 = tile_base(a.t, (unsigned long long)t);
         __syncthreads();   // the last tile's readers are done
@@ -356,11 +356,10 @@ __global__ void __launch_bounds__(kEvtThreads, 3) expval_tile_kernel(const float
                             w[i] = x + y;
                             w[i + h] = x - y;
                         }
-                float *rb = red + pb * 16 * kEvtThreads;
+                __syncthreads();   // the last group's entries have been read
 #pragma unroll
                 for (int i = 0; i < 16; ++i) rb[i * kEvtThreads + tid] = w[i];
                 __syncthreads();
-                // two buffers: a warp that writes the next one has read this one
                 for (int s = g.s0 + ((warp - g.s0) & 3); s < g.s1; s += 4) {
                     const EvtString &z = a.s[s];
                     const unsigned odd = (unsigned)(__popcll((b0 << 5) & z.z_out) & 1) ^ (r ? z.zr : 0u);
@@ -375,7 +374,6 @@ __global__ void __launch_bounds__(kEvtThreads, 3) expval_tile_kernel(const float
                     ff_add(f, pick_sign(sum, odd));
                     acc[s * 32 + lane] = make_float2(f.hi, f.lo);
                 }
-                pb ^= 1;
             }
         }
     }
@@ -400,7 +398,7 @@ __global__ void __launch_bounds__(128) expval_sum_kernel(const double *__restric
     if (threadIdx.x == 0) result[blockIdx.x] = (red[0] + red[1]) + (red[2] + red[3]);
 }
 
-constexpr int kEvtSmem = (8 << kEvtQubits) + 2 * 16 * kEvtThreads * (int)sizeof(float) + kEvtStrings * 32 * (int)sizeof(float2);
+constexpr int kEvtSmem = (8 << kEvtQubits) + 16 * kEvtThreads * (int)sizeof(float) + kEvtStrings * 32 * (int)sizeof(float2);
 
 // The tile pass of the strings order[..] listed in `runs` (each a run of equal x masks); res[i]
 // receives the i-th string's sum in the order of `placed`.
@@ -475,8 +473,8 @@ int launch_tiles(const float *sv, const EvtArgs &a, double *partials, double *re
             g_evt_attr |= bit;
         }
     }
-    const int grid = (int)std::min<long long>(a.tiles, 3ll * num_sms);
-    const int smem = (int)sizeof(float) * (64 << a.t.fb) + 2 * 16 * kEvtThreads * (int)sizeof(float) + a.n_strings * 32 * (int)sizeof(float2);
+    const int grid = (int)std::min<long long>(a.tiles, (long long)kEvtCtas * num_sms);
+    const int smem = (int)sizeof(float) * (64 << a.t.fb) + 16 * kEvtThreads * (int)sizeof(float) + a.n_strings * 32 * (int)sizeof(float2);
     expval_tile_kernel<<<grid, kEvtThreads, smem, s>>>(sv, a, partials);
     SV_CUDA_TRY(cudaGetLastError());
     expval_sum_kernel<<<a.n_strings, 128, 0, s>>>(partials, grid, a.n_strings, result);
@@ -515,7 +513,7 @@ extern "C" int sv_expval_pauli(const sv_state *st_c, const uint64_t *x_masks, co
         }
     // workspace: per-CTA partials for one launch, a counter, and one result per string
     const int max_grid = st->num_sms * 8;
-    const size_t n_partials = (size_t)st->num_sms * std::max(8 * kEvMaxStrings, 3 * kEvtStrings);
+    const size_t n_partials = (size_t)st->num_sms * std::max(8 * kEvMaxStrings, kEvtCtas * kEvtStrings);
     if (count > st->ev_capacity) {
         cudaStreamSynchronize(st->stream);
         cudaFree(st->d_ev);
