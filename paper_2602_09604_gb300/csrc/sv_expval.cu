@@ -283,12 +283,16 @@ int launch_ev(const float *sv, const EvArgs &a, double *partials, unsigned *coun
 // with different x masks, each a read of the whole state for the kernel above.  Here a CTA keeps a
 // tile -- 2^12 amplitudes agreeing on the qubits outside a local set that holds qubits 0-4 -- in
 // shared memory and evaluates every string whose x mask lies in the local set: per x mask (and
-// component) each thread forms 16 terms, takes their 16-point Walsh-Hadamard transform (every
-// sign pattern a z mask can put on the four index bits that vary in the thread), and each string sums
-// the 128 threads' entries for its mask, signed by its thread-index and tile parities.  z masks may
+// component) each thread forms 16 terms and takes two 8-point Walsh-Hadamard transforms (every sign
+// pattern a z mask can put on three of the four index bits that vary in the thread), and each string
+// adds the 128 threads' two entries for its mask, signed by the fourth bit and its thread-index and
+// tile parities, in float-float.  z masks may
 // name any qubit.  Terms of a pair (j, j ^ x) are equal once signed, so only one of each pair is formed.
 constexpr int kEvtThreads = 128;
 constexpr int kEvtQubits = 12;
+// From here on the two kernels' sums agree to 1e-9 (the rounding of the fp32 terms' sums averages out
+// with the number of terms: 4e-9 apart at 20 qubits); smaller states keep the one-mask kernel's sums.
+constexpr int kEvtMinQubits = 26;
 constexpr int kEvtCtas = 4;      // per SM: 53 KB of shared memory, 128 registers a thread
 constexpr int kEvtGroups = 32;
 constexpr int kEvtStrings = 64;
@@ -348,7 +352,7 @@ __global__ void __launch_bounds__(kEvtThreads, kEvtCtas) expval_tile_kernel(cons
                     w[i] = g.comp ? fmaf(vr, ui, -(vi * ur)) : fmaf(vr, ur, vi * ui);
                 }
 #pragma unroll
-                for (int h = 1; h < 16; h <<= 1)
+                for (int h = 1; h < 8; h <<= 1)   // two 8-point transforms: fp32 sums hold eight terms
 #pragma unroll
                     for (int i = 0; i < 16; ++i)
                         if (!(i & h)) {
@@ -363,15 +367,15 @@ __global__ void __launch_bounds__(kEvtThreads, kEvtCtas) expval_tile_kernel(cons
                 for (int s = g.s0 + ((warp - g.s0) & 3); s < g.s1; s += 4) {
                     const EvtString &z = a.s[s];
                     const unsigned odd = (unsigned)(__popcll((b0 << 5) & z.z_out) & 1) ^ (r ? z.zr : 0u);
-                    float sum = 0.f;
+                    const float2 v = acc[s * 32 + lane];
+                    FF2 f{v.x, v.y};
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const int e = lane + 32 * k;
-                        sum += pick_sign(rb[z.zw * kEvtThreads + e], (unsigned)__popc(e & z.zt) & 1u);
+                        const unsigned oe = odd ^ ((unsigned)__popc(e & z.zt) & 1u);
+                        ff_add(f, pick_sign(rb[(z.zw & 7) * kEvtThreads + e], oe));
+                        ff_add(f, pick_sign(rb[(8 + (z.zw & 7)) * kEvtThreads + e], oe ^ (z.zw >> 3)));
                     }
-                    const float2 v = acc[s * 32 + lane];
-                    FF2 f{v.x, v.y};
-                    ff_add(f, pick_sign(sum, odd));
                     acc[s * 32 + lane] = make_float2(f.hi, f.lo);
                 }
             }
@@ -546,7 +550,7 @@ extern "C" int sv_expval_pauli(const sv_state *st_c, const uint64_t *x_masks, co
         runs.push_back(EvRun{p, m});
         p += m;
     }
-    if (n >= kEvtQubits) {
+    if (n >= kEvtMinQubits) {
         while (!runs.empty()) {
             uint64_t lam = 31;
             int strings = 0, passes = 0;

@@ -47,3 +47,25 @@ def test_chain_terms_match_oracle(B, n):
     one = np.array([st.expval([t])[0] for t in strings])
     assert np.max(np.abs(one - got)) <= 40 * 2.0 ** -24
     st.free()
+
+
+def test_tiles_match_one_string_at_a_time(B):
+    """26 qubits, the smallest state whose strings share tile passes."""
+    import torch
+    from paper_2602_09604_gb300.state import DeviceState
+    n = 26
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    psi = torch.randn(1 << n, 2, device="cuda", generator=gen)
+    psi = (psi / torch.linalg.vector_norm(psi.double())).float().contiguous()
+    st = DeviceState(n)
+    B.sv_load(st.h, psi.data_ptr(), False)
+    strings = chain(n)
+    got = st.expval(strings)
+    assert np.array_equal(got, st.expval(strings))
+    one = np.array([st.expval([t])[0] for t in strings])
+    assert np.max(np.abs(one - got)) <= 40 * 2.0 ** -24
+    amps = torch.view_as_complex(psi).to(torch.complex128)
+    probs = amps.abs().square().view(-1, 4096)
+    sign = torch.tensor([(-1.0) ** bin(i & 3).count("1") for i in range(4096)], dtype=torch.float64, device="cuda")
+    assert abs(got[strings.index({0: "Z", 1: "Z"})] - float((probs * sign).sum())) <= 20 * 2.0 ** -24
+    st.free()
