@@ -1011,10 +1011,23 @@ int apply_core(sv_state *st, sv_fused *f, sv_timing *timings, const std::vector<
         }
         return launch_fused_gate(st->d, st->n, g, device_mats(i), device_tc(i), st->stream, st->num_sms);
     };
-    if (!timings && !st->c128) {
+    sv_fused::Plan *pl = &f->plans[m > 0 ? 1 : 0];
+    bool planned = !timings && !st->c128;
+    if (planned && !pl->ready) {
+        // The plan's images are uploaded once.  On a stream that is being captured nothing may be
+        // uploaded, and without device memory nothing can be: such a call launches gate by gate.
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        const cudaError_t ce = cudaStreamIsCapturing(st->stream, &cap);
+        if (ce != cudaSuccess) cudaGetLastError();
+        planned = ce == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
+                  ensure_plan(f, pl, m > 0 ? lazy : nullptr, A, a, st->device) == SV_OK;
+        if (!planned) {
+            cudaGetLastError();
+            clear_error();
+        }
+    }
+    if (planned) {
         // no record per gate is asked for: gates go in passes (the plan; see sv_stage.cu)
-        sv_fused::Plan *pl = &f->plans[m > 0 ? 1 : 0];
-        rc = ensure_plan(f, pl, m > 0 ? lazy : nullptr, A, a, st->device);
         for (size_t s = 0; rc == SV_OK && s < pl->small.steps.size(); ++s) {
             const PassStep &ps = pl->small.steps[s];
             if (ps.single < 0) rc = launch_stage(small, pl->d_plan, ps, st->stream, st->num_sms);

@@ -90,3 +90,35 @@ def test_tensor_core_circuits_keep_order_and_bits(B, n):
     got, one = run(B, n, f, psi=psi), run(B, n, f, psi=psi, timings=True)
     assert np.array_equal(got.view(np.uint64), one.view(np.uint64))
     B.sv_fused_free(f)
+
+
+@pytest.mark.parametrize("warm", [False, True])
+def test_apply_in_a_captured_graph(B, warm):
+    """Captured before any plan exists (one launch per gate) and after (passes): replays give the
+    same state as an ordinary call."""
+    import torch
+    from paper_2602_09604_gb300.state import DeviceState
+    n = 13
+    gates = circuit(n, 3, seed=77)
+    f = B.sv_fuse_circuit(gates, n, max_k=3)
+    tol = 2 * bound(B, f)
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        st = DeviceState(n, stream=s)
+        if warm:
+            st.init(0)
+            st.apply(f)
+        s.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            st.apply(f)
+        st.init(5)
+        graph.replay()
+        s.synchronize()
+        got = st.store()
+        st.init(5)
+        st.apply(f, timings=True)
+        want = st.store()
+    assert oracle.l2_error(want.astype(np.complex128), got) <= tol
+    st.free()
+    B.sv_fused_free(f)
