@@ -242,8 +242,12 @@ SV_API int sv_fused_get_matrix(const sv_fused *f, int i, double *out);
 
 /* Apply every fused gate, in order, to the state (Eq. 3 per fused gate).  The first call with a
  * given fused circuit uploads the matrices that do not travel as kernel arguments (k = 6 and the
- * tensor-core operands) with cudaMalloc/cudaMemcpy.  With `timings` non-NULL (one record per
- * fused gate) each launch is bracketed by CUDA events and the call synchronises. */
+ * tensor-core operands) with cudaMalloc/cudaMemcpy.  Without `timings`, CUDA-core fp32 gates whose
+ * qubits lie close together share passes over the state (a gate only moves ahead of gates on other
+ * qubits; the plan and its matrices are made and uploaded on the first such call, and a call on a
+ * stream that is being captured before that launches gate by gate).  With `timings` non-NULL (one
+ * record per fused gate) every gate has its own launch, bracketed by CUDA events, and the call
+ * synchronises. */
 SV_API int sv_apply_fused_gates(sv_state *st, const sv_fused *f, sv_timing *timings);
 
 /* ---------------------------------------------------------------------------------------------
@@ -345,7 +349,8 @@ SV_API int sv_alloc_c128(int n_qubits, void *dev_ptr, size_t bytes, void *cuda_s
  * state is not normalised first (divide by sv_norm for a state that is not unit-norm).  Each
  * amplitude's term is formed in fp32 and accumulated in float-float per thread, fp64 across
  * threads, in a fixed order (deterministic).  Strings sharing an x mask share read passes, up to 8
- * strings per pass over the 8 * 2^n bytes.  SV_EINVAL if a mask has a bit >= n.  Grows a small
+ * strings per pass over the 8 * 2^n bytes; on states of 26 or more qubits strings with different x masks
+ * share passes too (up to 64 strings whose x masks touch at most 7 qubits above qubit 4).  SV_EINVAL if a mask has a bit >= n.  Grows a small
  * workspace on the state's device when count exceeds the previous maximum.  Synchronises. */
 SV_API int sv_expval_pauli(const sv_state *st, const uint64_t *x_masks, const uint64_t *z_masks, int count, double *out);
 
