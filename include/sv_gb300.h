@@ -247,7 +247,11 @@ SV_API int sv_fused_get_matrix(const sv_fused *f, int i, double *out);
  * qubits; the plan and its matrices are made and uploaded on the first such call, and a call on a
  * stream that is being captured before that launches gate by gate).  With `timings` non-NULL (one
  * record per fused gate) every gate has its own launch, bracketed by CUDA events, and the call
- * synchronises. */
+ * synchronises.
+ *
+ * A graph captured from a call (also of sv_init_apply) keeps the shared passes' matrices alive by
+ * itself: it may be replayed after sv_fused_free.  Matrices of k = 6 gates and tensor-core operands
+ * belong to the fused circuit: a graph with such gates is replayed only while the circuit exists. */
 SV_API int sv_apply_fused_gates(sv_state *st, const sv_fused *f, sv_timing *timings);
 
 /* ---------------------------------------------------------------------------------------------

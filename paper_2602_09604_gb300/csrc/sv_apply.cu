@@ -876,27 +876,26 @@ int ensure_plan(sv_fused *f, sv_fused::Plan *pl, const std::vector<char> *lazy, 
     pl->rest_off = ns;
     const size_t bytes = (ns + nr) * sizeof(float);
     if (bytes > 0) {
-        void *buf = nullptr;
-        size_t got = 0;
-        SV_TRY(dev_buffer_get(device, bytes, &buf, &got));
+        SharedBuffer *buf = nullptr;
+        SV_TRY(shared_buffer_get(device, bytes, &buf));
         std::unique_lock<std::mutex> lk;
         unsigned char *img = nullptr;
         int rc = pinned_staging(bytes, &img, lk);
         if (rc == SV_OK) {
             if (ns) std::memcpy(img, pl->small.image.data(), ns * sizeof(float));
             if (nr) std::memcpy(img + ns * sizeof(float), pl->rest.image.data(), nr * sizeof(float));
-            const cudaError_t e = cudaMemcpy(buf, img, bytes, cudaMemcpyHostToDevice);
+            const cudaError_t e = cudaMemcpy(buf->p, img, bytes, cudaMemcpyHostToDevice);
             if (e != cudaSuccess) {
                 set_error("sv_apply_fused_gates: pass images: %s", cudaGetErrorString(e));
                 rc = SV_ECUDA;
             }
         }
         if (rc != SV_OK) {
-            dev_buffer_put(device, buf, got);
+            shared_buffer_release(buf);
             return rc;
         }
-        pl->d_plan = static_cast<float *>(buf);
-        pl->d_plan_bytes = got;
+        pl->buf = buf;
+        pl->d_plan = static_cast<float *>(buf->p);
         pl->small.image = std::vector<float>();
         pl->rest.image = std::vector<float>();
     }
@@ -918,6 +917,11 @@ int apply_core(sv_state *st, sv_fused *f, sv_timing *timings, const std::vector<
                 return SV_EINVAL;
             }
     std::lock_guard<std::mutex> use(f->mu);
+    // (a stream whose state cannot be read is taken as captured: its launches report the error)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const cudaError_t cap_error = cudaStreamIsCapturing(st->stream, &cap);
+    if (cap_error != cudaSuccess) cudaGetLastError();
+    const bool capturing = cap_error != cudaSuccess || cap != cudaStreamCaptureStatusNone;
     if (st->c128) SV_TRY(upload_fused_c128(f, st->device));
     else SV_TRY(upload_fused(f, st->device));
     const size_t ng = f->gates.size();
@@ -1013,14 +1017,12 @@ int apply_core(sv_state *st, sv_fused *f, sv_timing *timings, const std::vector<
     };
     sv_fused::Plan *pl = &f->plans[m > 0 ? 1 : 0];
     bool planned = !timings && !st->c128;
-    if (planned && !pl->ready) {
+    if (planned && (!pl->ready || capturing)) {
         // The plan's images are uploaded once.  On a stream that is being captured nothing may be
-        // uploaded, and without device memory nothing can be: such a call launches gate by gate.
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        const cudaError_t ce = cudaStreamIsCapturing(st->stream, &cap);
-        if (ce != cudaSuccess) cudaGetLastError();
-        planned = ce == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
-                  ensure_plan(f, pl, m > 0 ? lazy : nullptr, A, a, st->device) == SV_OK;
+        // uploaded, and without device memory nothing can be: such a call launches gate by gate.  A
+        // capture that uses them makes its graph one of their owners.
+        planned = capturing ? pl->ready && (!pl->buf || shared_buffer_retain_in_capture(pl->buf, st->stream) == SV_OK)
+                            : ensure_plan(f, pl, m > 0 ? lazy : nullptr, A, a, st->device) == SV_OK;
         if (!planned) {
             cudaGetLastError();
             clear_error();
@@ -1070,6 +1072,7 @@ int apply_core(sv_state *st, sv_fused *f, sv_timing *timings, const std::vector<
             rc = SV_ETIMEOUT;
         }
     }
+    if (capturing) return rc;   // nothing was launched, and the stream's event stays with its last launch
     const int urc = note_fused_use(f, st->stream);   // even after an error: launches may be queued
     return rc != SV_OK ? rc : urc;
 }
@@ -1138,9 +1141,10 @@ extern "C" int sv_device_status(void)
 extern "C" void sv_fused_free(sv_fused *f)
 {
     if (!f) return;
-    if (f->d_buf || f->d_mats64 || !f->use_events.empty()) {
+    if (f->d_buf || f->d_mats64 || f->plans[0].buf || f->plans[1].buf || !f->use_events.empty()) {
         // only the streams that applied this circuit can still read its images: wait for each
-        // one's last launch (its event), then return the buffers to the library's cache
+        // one's last launch (its event), then return the buffers to the library's cache (pass
+        // images that a captured graph holds go there with the graph)
         int cur = -1;
         cudaGetDevice(&cur);
         if (f->device >= 0 && cur != f->device) cudaSetDevice(f->device);
@@ -1151,7 +1155,8 @@ extern "C" void sv_fused_free(sv_fused *f)
         f->use_events.clear();
         dev_buffer_put(f->device, f->d_buf, f->d_buf_bytes);
         dev_buffer_put(f->device, f->d_mats64, f->d_mats64_bytes);
-        for (sv_fused::Plan &p : f->plans) dev_buffer_put(f->device, p.d_plan, p.d_plan_bytes);
+        for (sv_fused::Plan &p : f->plans) shared_buffer_release(p.buf);
+        shared_buffers_collect();
         if (f->device >= 0 && cur >= 0 && cur != f->device) cudaSetDevice(cur);
     }
     delete f;

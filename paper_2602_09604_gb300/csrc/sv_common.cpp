@@ -5,6 +5,7 @@
 #include <cstdio>
 #include <future>
 #include <mutex>
+#include <new>
 #include <system_error>
 #include <thread>
 
@@ -21,12 +22,74 @@ std::mutex g_buf_mu;
 std::vector<DevBuf> g_buf_cache[64];
 constexpr size_t kBufCacheCount = 8;
 constexpr size_t kBufCacheBytes = size_t(256) << 20;
+SharedBuffer *g_dropped = nullptr;   // shared buffers without an owner, not yet back in the cache
+
+// A graph that held a buffer has been destroyed, or never took it over: called by the driver on a
+// thread of its own, where no CUDA call is allowed.
+void release_from_graph(void *b) { shared_buffer_release(static_cast<SharedBuffer *>(b)); }
 }  // namespace
+
+int shared_buffer_get(int device, size_t bytes, SharedBuffer **out)
+{
+    *out = nullptr;
+    SharedBuffer *b = new (std::nothrow) SharedBuffer;
+    if (!b) { set_error("out of host memory"); return SV_ENOMEM; }
+    b->device = device;
+    const int rc = dev_buffer_get(device, bytes, &b->p, &b->bytes);
+    if (rc != SV_OK) {
+        delete b;
+        return rc;
+    }
+    *out = b;
+    return SV_OK;
+}
+
+void shared_buffer_release(SharedBuffer *b)
+{
+    if (!b || b->owners.fetch_sub(1) != 1) return;
+    std::lock_guard<std::mutex> lk(g_buf_mu);
+    b->next = g_dropped;
+    g_dropped = b;
+}
+
+void shared_buffers_collect()
+{
+    SharedBuffer *b = nullptr;
+    {
+        std::lock_guard<std::mutex> lk(g_buf_mu);
+        std::swap(b, g_dropped);
+    }
+    while (b) {
+        SharedBuffer *next = b->next;
+        dev_buffer_put(b->device, b->p, b->bytes);
+        delete b;
+        b = next;
+    }
+}
+
+int shared_buffer_retain_in_capture(SharedBuffer *b, cudaStream_t stream)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    cudaGraph_t graph = nullptr;
+    SV_CUDA_TRY(cudaStreamGetCaptureInfo(stream, &st, nullptr, &graph, nullptr, nullptr, nullptr));
+    if (st != cudaStreamCaptureStatusActive || !graph) { set_error("stream is not being captured"); return SV_ESTATE; }
+    cudaUserObject_t obj = nullptr;
+    SV_CUDA_TRY(cudaUserObjectCreate(&obj, b, release_from_graph, 1, cudaUserObjectNoDestructorSync));
+    b->owners.fetch_add(1);   // the object's; its end releases it
+    const cudaError_t e = cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove);
+    if (e != cudaSuccess) {
+        cudaUserObjectRelease(obj, 1);
+        set_error("keeping a buffer with a captured graph: %s", cudaGetErrorString(e));
+        return SV_ECUDA;
+    }
+    return SV_OK;
+}
 
 int dev_buffer_get(int device, size_t bytes, void **out, size_t *got_bytes)
 {
     *out = nullptr;
     *got_bytes = 0;
+    shared_buffers_collect();
     if (device >= 0 && device < 64) {
         std::lock_guard<std::mutex> lk(g_buf_mu);
         std::vector<DevBuf> &c = g_buf_cache[device];

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <complex>
 #include <cstdint>
 #include <functional>
@@ -157,6 +158,24 @@ int pinned_staging(size_t bytes, unsigned char **out, std::unique_lock<std::mute
 // and frees what the cache does not keep (at most 8 buffers, 256 MB per device).
 int dev_buffer_get(int device, size_t bytes, void **out, size_t *got_bytes);
 void dev_buffer_put(int device, void *p, size_t bytes);
+// A buffer of that cache with more than one owner: a fused circuit's pass images belong to the
+// circuit and to every graph captured from it, so a graph can be replayed after the circuit is
+// freed.  The last release puts it aside without a CUDA call (a graph's end may be reported where
+// none is allowed); shared_buffers_collect, called by dev_buffer_get too, puts such buffers back into
+// the cache.
+struct SharedBuffer {
+    std::atomic<int> owners{1};
+    int device = -1;
+    void *p = nullptr;
+    size_t bytes = 0;
+    SharedBuffer *next = nullptr;
+};
+int shared_buffer_get(int device, size_t bytes, SharedBuffer **out);
+void shared_buffer_release(SharedBuffer *b);
+void shared_buffers_collect();
+// Makes the graph that `stream` is being captured into an owner (and with it every executable graph
+// made from it, until its last replay has ended).
+int shared_buffer_retain_in_capture(SharedBuffer *b, cudaStream_t stream);
 // A gate's inputs read from another buffer: input amplitude i is src[offset(i) - off] when
 // (i & mask) == rest and 0 otherwise (offset = the blocked-layout float offset); the outputs still
 // cover the whole state.  Used for the first full-state gate after a lazy start: src is the small
@@ -246,8 +265,8 @@ struct sv_fused {
         std::vector<int> small_index, rest_index;  // their and the other gates' indices, in order
         svg::PassPlan small, rest;
         size_t rest_off = 0;                       // floats into d_plan of the second part's image
-        float *d_plan = nullptr;                   // both images (released with the circuit)
-        size_t d_plan_bytes = 0;
+        svg::SharedBuffer *buf = nullptr;          // both images, shared with graphs captured from the circuit
+        float *d_plan = nullptr;                   // = buf's memory
     };
     Plan plans[2];
     std::mutex mu;                                 // uploads, plans and use_events
