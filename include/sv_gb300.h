@@ -494,6 +494,7 @@ SV_API int sv_device_status(void);
  * callers that cannot afford the device-wide synchronisation cudaMalloc/cudaFree may cause.
  *
  * dev_state: the blocked-layout state of an n-qubit register (as sv_alloc would wrap), read only.
+ * It may lie at any float boundary (SV_EINVAL otherwise); from 16-byte boundaries it is read by wider loads.
  * n_qubits <= 30 and n_samples <= 4096 (the fixed array's limits; larger requests return
  * SV_EINVAL with a message).  uniforms / out: host arrays as in sv_sample.  Work is enqueued on
  * cuda_stream on the current device, and the call synchronises that stream before returning.

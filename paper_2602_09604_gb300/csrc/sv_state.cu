@@ -160,16 +160,26 @@ constexpr int kChunkThreads = 256;
 
 __device__ __forceinline__ double ff_value(const FF &a) { return (double)a.hi + (double)a.lo; }
 
+// Four floats by one 16-byte load, or (V4 false: a state given to sv_sample_noalloc need not be
+// aligned to more than its floats) by four loads.
+template <bool V4>
+__device__ __forceinline__ float4 load4(const float *p)
+{
+    if constexpr (V4) return *reinterpret_cast<const float4 *>(p);
+    else return make_float4(p[0], p[1], p[2], p[3]);
+}
+
 // |re|^2 + |im|^2 of `items` 16-byte pairs (item i: block i >> 3, quarter i & 7) of the blocks at
 // `base`, taken first, first + step, ...: a chain each for the real and the imaginary parts
+template <bool V4>
 __device__ __forceinline__ double sum_items(const float *__restrict__ base, int first, int step, int items)
 {
     FF re{0.f, 0.f}, im{0.f, 0.f};
 #pragma unroll 8
     for (int i = first; i < items; i += step) {
         const float *b = base + (i >> 3) * 64 + (i & 7) * 4;
-        const float4 r = *reinterpret_cast<const float4 *>(b);
-        const float4 m = *reinterpret_cast<const float4 *>(b + 32);
+        const float4 r = load4<V4>(b);
+        const float4 m = load4<V4>(b + 32);
         ff_add_sq(re, r.x); ff_add_sq(im, m.x);
         ff_add_sq(re, r.y); ff_add_sq(im, m.y);
         ff_add_sq(re, r.z); ff_add_sq(im, m.z);
@@ -178,11 +188,12 @@ __device__ __forceinline__ double sum_items(const float *__restrict__ base, int 
     return ff_value(re) + ff_value(im);
 }
 
+template <bool V4>
 __global__ void __launch_bounds__(kChunkThreads) chunk_sum_kernel(const float *__restrict__ sv, int chunk_blocks_log2,
                                                                   double *__restrict__ chunk_sum)
 {
     __shared__ double ws[kChunkThreads / 32];
-    const double v = warp_sum_d(sum_items(sv + ((long long)blockIdx.x << chunk_blocks_log2) * 64, (int)threadIdx.x, kChunkThreads,
+    const double v = warp_sum_d(sum_items<V4>(sv + ((long long)blockIdx.x << chunk_blocks_log2) * 64, (int)threadIdx.x, kChunkThreads,
                                           8 << chunk_blocks_log2));
     if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
     __syncthreads();
@@ -248,6 +259,7 @@ __global__ void __launch_bounds__(1024) chunk_scan_kernel(const double *__restri
 constexpr int kSearchThreads = 256;
 constexpr int kSearchStep = 8 * kSearchThreads;
 
+template <bool V4>
 __global__ void __launch_bounds__(kSearchThreads) sample_search_kernel(const float *__restrict__ sv, int n, long long n_chunks,
                                                                        int chunk_log2, const double *__restrict__ prefix,
                                                                        const double *__restrict__ uniforms, int n_samples,
@@ -274,7 +286,7 @@ __global__ void __launch_bounds__(kSearchThreads) sample_search_kernel(const flo
     double run = prefix[lo];
     if (chunk_log2 == kChunkLog2) {
         constexpr int kItems = (1 << kChunkLog2) / 4 / (kSearchThreads / 32);   // a warp's 16-byte pairs
-        const double v = warp_sum_d(sum_items(sv + (long long)(i0 >> 5) * 64 + (long long)warp * kItems * 8, lane, 32, kItems));
+        const double v = warp_sum_d(sum_items<V4>(sv + (long long)(i0 >> 5) * 64 + (long long)warp * kItems * 8, lane, 32, kItems));
         if (lane == 0) part[warp] = v;
         __syncthreads();
         int p = 0;   // every thread: the same sums in the same order
@@ -290,8 +302,8 @@ __global__ void __launch_bounds__(kSearchThreads) sample_search_kernel(const flo
         const bool in = i < N;   // N < 8 (n < 3): the block is zero-padded, and the answer is clamped
         if (in) {
             const float *b = sv + re_off(i);
-            const float4 r0 = *reinterpret_cast<const float4 *>(b), r1 = *reinterpret_cast<const float4 *>(b + 4);
-            const float4 m0 = *reinterpret_cast<const float4 *>(b + 32), m1 = *reinterpret_cast<const float4 *>(b + 36);
+            const float4 r0 = load4<V4>(b), r1 = load4<V4>(b + 4);
+            const float4 m0 = load4<V4>(b + 32), m1 = load4<V4>(b + 36);
             const float re[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
             const float im[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
 #pragma unroll
@@ -546,12 +558,12 @@ int sample_impl(sv_state *st, const double *uniforms, int n_samples, uint64_t *o
     if (st->c128) {
         SV_TRY(c128_sample(st, n_samples));
     } else {
-        chunk_sum_kernel<<<(unsigned)nc, kChunkThreads, 0, st->stream>>>(st->d, chunk_blocks_log2, sums);
+        chunk_sum_kernel<true><<<(unsigned)nc, kChunkThreads, 0, st->stream>>>(st->d, chunk_blocks_log2, sums);
         SV_CUDA_TRY(cudaGetLastError());
         chunk_scan_kernel<<<1, 1024, 0, st->stream>>>(sums, prefix, nc);
         SV_CUDA_TRY(cudaGetLastError());
         if (n_samples > 0) {
-            sample_search_kernel<<<n_samples, kSearchThreads, 0, st->stream>>>(st->d, n, nc, chunk_log2, prefix, st->d_uniforms,
+            sample_search_kernel<true><<<n_samples, kSearchThreads, 0, st->stream>>>(st->d, n, nc, chunk_log2, prefix, st->d_uniforms,
                                                                                  n_samples, st->d_samples);
             SV_CUDA_TRY(cudaGetLastError());
         }
@@ -631,6 +643,7 @@ extern "C" int sv_sample_noalloc(const void *dev_state, int n_qubits, void *cuda
         return SV_EINVAL;
     }
     if (n_samples == 0) return SV_OK;
+    if (reinterpret_cast<uintptr_t>(dev_state) % sizeof(float)) { set_error("sv_sample_noalloc: dev_state is not aligned to its floats"); return SV_EINVAL; }
     for (int s = 0; s < n_samples; ++s)
         if (!(uniforms[s] >= 0.0 && uniforms[s] < 1.0)) { set_error("sv_sample_noalloc: uniform %d = %g is not in [0, 1)", s, uniforms[s]); return SV_EINVAL; }
     int device = 0;
@@ -647,11 +660,13 @@ extern "C" int sv_sample_noalloc(const void *dev_state, int n_qubits, void *cuda
     unsigned long long *d_out = reinterpret_cast<unsigned long long *>(d_u + kNoAllocMaxSamples);
     const float *sv = static_cast<const float *>(dev_state);
     SV_CUDA_TRY(cudaMemcpyAsync(d_u, uniforms, sizeof(double) * size_t(n_samples), cudaMemcpyHostToDevice, stream));
-    chunk_sum_kernel<<<(unsigned)nc, kChunkThreads, 0, stream>>>(sv, chunk_log2 - 5, sums);
+    const bool v4 = reinterpret_cast<uintptr_t>(dev_state) % 16 == 0;
+    (v4 ? chunk_sum_kernel<true> : chunk_sum_kernel<false>)<<<(unsigned)nc, kChunkThreads, 0, stream>>>(sv, chunk_log2 - 5, sums);
     SV_CUDA_TRY(cudaGetLastError());
     chunk_scan_kernel<<<1, 1024, 0, stream>>>(sums, prefix, nc);
     SV_CUDA_TRY(cudaGetLastError());
-    sample_search_kernel<<<n_samples, kSearchThreads, 0, stream>>>(sv, n, nc, chunk_log2, prefix, d_u, n_samples, d_out);
+    (v4 ? sample_search_kernel<true> : sample_search_kernel<false>)<<<n_samples, kSearchThreads, 0, stream>>>(sv, n, nc, chunk_log2, prefix, d_u,
+                                                                                                            n_samples, d_out);
     SV_CUDA_TRY(cudaGetLastError());
     SV_CUDA_TRY(cudaMemcpyAsync(out, d_out, sizeof(unsigned long long) * size_t(n_samples), cudaMemcpyDeviceToHost, stream));
     SV_CUDA_TRY(cudaStreamSynchronize(stream));
