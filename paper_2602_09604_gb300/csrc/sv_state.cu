@@ -216,6 +216,14 @@ __device__ __forceinline__ double warp_scan_d(double v, int lane)
     return v;
 }
 
+// the sum before this lane, from its inclusive scan (a difference incl - own would lose what is
+// small against the lane's own value)
+__device__ __forceinline__ double warp_before_d(double incl, int lane)
+{
+    const double t = __shfl_up_sync(0xffffffffu, incl, 1);
+    return lane ? t : 0.0;
+}
+
 // single CTA exclusive scan of n chunk sums (in: sums, out: prefix), total at prefix[n]:
 // each thread sums its own range, the 1024 range sums are scanned by warps, then each thread writes
 // its range
@@ -241,7 +249,7 @@ __global__ void __launch_bounds__(1024) chunk_scan_kernel(const double *__restri
         }
     }
     __syncthreads();
-    double run = (incl - s) + (warp ? seg[warp - 1] : 0.0);
+    double run = warp_before_d(incl, lane) + (warp ? seg[warp - 1] : 0.0);
 #pragma unroll 8
     for (long long i = lo; i < hi; ++i) {
         prefix[i] = run;
@@ -313,6 +321,7 @@ __global__ void __launch_bounds__(kSearchThreads) sample_search_kernel(const flo
             }
         }
         const double incl = warp_scan_d(own, lane);
+        const double lane_before = warp_before_d(incl, lane);
         if (lane == 31) part[warp] = incl;
         if (threadIdx.x == 0) s_first = kSearchThreads;
         __syncthreads();
@@ -328,7 +337,7 @@ __global__ void __launch_bounds__(kSearchThreads) sample_search_kernel(const flo
         const int first = s_first;
         if (first < kSearchThreads) {
             if ((int)threadIdx.x == first) {
-                double t = before + (incl - own);
+                double t = before + lane_before;
                 int e = 0;
 #pragma unroll
                 for (int q = 0; q < 7; ++q)
