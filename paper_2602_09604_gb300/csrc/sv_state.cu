@@ -188,6 +188,60 @@ __device__ __forceinline__ double sum_items(const float *__restrict__ base, int 
     return ff_value(re) + ff_value(im);
 }
 
+// s = a + b, err = what the rounding left out (two-sum)
+__device__ __forceinline__ float two_sum(float a, float b, float &err)
+{
+    const float s = a + b;
+    const float bp = s - a;
+    err = (a - (s - bp)) + (b - bp);
+    return s;
+}
+
+// The same sum to fp64's rounding, by one warp.  fp64 multiply-adds run at 2 a clock on an SM, so the
+// squares are added as three floats: p and its remainder are exact for factors of 2^-50 to 2^60, what
+// the first two floats round off goes to the third (relative error below 2^-60, before the last fp64
+// additions; float-float left 2^-42).  A warp that meets another factor adds in fp64.
+// A 20-qubit state, whole call with 1024 / 4096 samples: 99 / 227 us; in fp64 203 / 635; float-float 100 / 228.
+template <bool V4>
+__device__ __forceinline__ double warp_sum_items_exact(const float *__restrict__ base, int lane, int items)
+{
+    constexpr unsigned kLow = (127u - 50u) << 23, kHigh = (127u + 60u) << 23;   // as float bits
+    float hi = 0.f, lo = 0.f, rest = 0.f;
+    bool other = false;
+    auto add = [&](float v) {
+        const unsigned u = __float_as_uint(v) & 0x7fffffffu;
+        other |= u != 0u && u - kLow > kHigh - kLow;
+        const float p = v * v, ep = fmaf(v, v, -p);
+        float e, e2, e3;
+        hi = two_sum(hi, p, e);
+        lo = two_sum(lo, e, e2);
+        lo = two_sum(lo, ep, e3);
+        rest += e2 + e3;
+    };
+#pragma unroll 4
+    for (int i = lane; i < items; i += 32) {
+        const float *b = base + (i >> 3) * 64 + (i & 7) * 4;
+        const float4 r = load4<V4>(b);
+        const float4 m = load4<V4>(b + 32);
+        add(r.x); add(r.y); add(r.z); add(r.w);
+        add(m.x); add(m.y); add(m.z); add(m.w);
+    }
+    double v = (double)hi + ((double)lo + (double)rest);
+    if (__any_sync(0xffffffffu, other)) {
+        double re = 0.0, im = 0.0;
+        for (int i = lane; i < items; i += 32) {
+            const float *b = base + (i >> 3) * 64 + (i & 7) * 4;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                re = fma((double)b[e], (double)b[e], re);
+                im = fma((double)b[e + 32], (double)b[e + 32], im);
+            }
+        }
+        v = re + im;
+    }
+    return warp_sum_d(v);
+}
+
 template <bool V4>
 __global__ void __launch_bounds__(kChunkThreads) chunk_sum_kernel(const float *__restrict__ sv, int chunk_blocks_log2,
                                                                   double *__restrict__ chunk_sum)
@@ -259,9 +313,8 @@ __global__ void __launch_bounds__(1024) chunk_scan_kernel(const double *__restri
 
 // One CTA per sample; p_i = re^2 + im^2 in fp64 (products of widened floats are exact).  The chunk
 // holding the sample is found by 256 probes of the chunk prefix sums at a time; each warp sums an
-// eighth of a full chunk (float-float: fp64 multiply-adds run at 2 a clock on an SM, and 16 K of them
-// a sample were the call's longest part); the eighth where the running total passes the target is
-// then walked 2048 amplitudes at a step, eight to a thread, with a scan over the CTA, to the first
+// eighth of a full chunk to fp64's rounding; the eighth where the running total passes the target is then
+// walked 2048 amplitudes at a step, eight to a thread, with a scan over the CTA, to the first
 // index whose running total exceeds it, going on past the eighth if rounding leaves the target
 // just past its end.
 constexpr int kSearchThreads = 256;
@@ -293,8 +346,10 @@ __global__ void __launch_bounds__(kSearchThreads) sample_search_kernel(const flo
     unsigned long long i0 = (unsigned long long)lo << chunk_log2;
     double run = prefix[lo];
     if (chunk_log2 == kChunkLog2) {
-        constexpr int kItems = (1 << kChunkLog2) / 4 / (kSearchThreads / 32);   // a warp's 16-byte pairs
-        const double v = warp_sum_d(sum_items<V4>(sv + (long long)(i0 >> 5) * 64 + (long long)warp * kItems * 8, lane, 32, kItems));
+        // 16-byte pairs of a warp; the last eighth's sum decides nothing
+        constexpr int kItems = (1 << kChunkLog2) / 4 / (kSearchThreads / 32);
+        double v = 0.0;
+        if (warp < kSearchThreads / 32 - 1) v = warp_sum_items_exact<V4>(sv + (long long)(i0 >> 5) * 64 + (long long)warp * kItems * 8, lane, kItems);
         if (lane == 0) part[warp] = v;
         __syncthreads();
         int p = 0;   // every thread: the same sums in the same order
