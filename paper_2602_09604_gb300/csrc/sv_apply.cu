@@ -865,9 +865,11 @@ int ensure_plan(sv_fused *f, sv_fused::Plan *pl, const std::vector<char> *lazy, 
         }
     }
     for (const FusedGate &g : pl->small_gates) small.push_back(&g);
+    bool keep_order = false;   // by the circuit's own paths: neither part may be reordered ahead of the other's tensor-core gates
+    for (const FusedGate &g : f->gates) keep_order |= g.path == SV_PATH_TC_TF32 || g.path == SV_PATH_TC_BF16X3;
     try {
-        plan_passes(small, a, &pl->small);
-        plan_passes(rest, f->n, &pl->rest);
+        plan_passes(small, a, keep_order, &pl->small);
+        plan_passes(rest, f->n, keep_order, &pl->rest);
     } catch (const std::exception &) {
         set_error("sv_apply_fused_gates: out of host memory for the launch plan");
         return SV_ENOMEM;

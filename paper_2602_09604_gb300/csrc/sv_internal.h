@@ -138,9 +138,10 @@ struct PassPlan {
     std::vector<float> image;   // the passes' descriptors and matrices (16-byte multiples), one after another
 };
 // Cuts gates (in circuit order, on an n-qubit state) into passes and single launches.  Gates move
-// ahead only of gates on other qubits, and not at all in a circuit with tensor-core gates (their
-// operand split turns a last-bit difference of the input into a larger one).
-void plan_passes(const std::vector<const FusedGate *> &gates, int n, PassPlan *plan);
+// ahead only of gates on other qubits, and with keep_order not at all: a circuit with a tensor-core
+// gate anywhere keeps its order (the operand split turns a last-bit difference of the input into a
+// larger one).
+void plan_passes(const std::vector<const FusedGate *> &gates, int n, bool keep_order, PassPlan *plan);
 int launch_stage(float *sv, const float *image, const PassStep &p, cudaStream_t stream, int num_sms);
 
 // Tensor-core path (sv_tc.cu): host-side operand images and the launcher.

@@ -9,7 +9,9 @@
 // written once per pass instead of once per gate.
 //
 // A gate joins a pass when no earlier gate left out shares a qubit with it, so it only moves ahead
-// of gates on other qubits (exact).  Every output is formed by the same chain of fused multiply-adds
+// of gates on other qubits: the same product, but its roundings fall in another order (96
+// Grover circuits of 10 to 25 qubits: errors of 0.25 to 4 times those in circuit order, 0.93 in the
+// geometric mean; grids and quantum volume 0.98 to 1.04).  Every output is formed by the same chain of fused multiply-adds
 // as in the one-gate kernels (columns in order; re += ar xr, re -= ai xi, im += ar xi, im += ai xr),
 // so passes that keep the circuit's order give the same bits.
 //
@@ -321,15 +323,14 @@ void fill_stage(const std::vector<const FusedGate *> &gates, const std::vector<i
 
 }  // namespace
 
-void plan_passes(const std::vector<const FusedGate *> &gates, int n, PassPlan *plan)
+void plan_passes(const std::vector<const FusedGate *> &gates, int n, bool keep_order, PassPlan *plan)
 {
     plan->steps.clear();
     plan->image.clear();
     std::vector<int> left;
-    bool reorder = true, small = true;
+    bool small = true;
     for (size_t i = 0; i < gates.size(); ++i) {
         left.push_back((int)i);
-        if (gates[i]->path == SV_PATH_TC_TF32 || gates[i]->path == SV_PATH_TC_BF16X3) reorder = false;
         if (gates[i]->k > 2) small = false;
     }
     // Large tiles hold more gates a pass; on a small state they leave SMs without a tile, and a pass is
@@ -362,7 +363,7 @@ void plan_passes(const std::vector<const FusedGate *> &gates, int n, PassPlan *p
             }
             blocked |= q;
             rest.push_back(left[s]);
-            if (!reorder) {
+            if (keep_order) {
                 rest.insert(rest.end(), left.begin() + (long)s + 1, left.end());
                 break;
             }
