@@ -254,6 +254,22 @@ SV_API int sv_fused_get_matrix(const sv_fused *f, int i, double *out);
  * belong to the fused circuit: a graph with such gates is replayed only while the circuit exists. */
 SV_API int sv_apply_fused_gates(sv_state *st, const sv_fused *f, sv_timing *timings);
 
+/* The launches that a call without timing records makes of f's gates on a complex64 state, in order --
+ * host only, no GPU: sv_apply_fused_gates, or (from_basis != 0) sv_init_apply.  Returns their number L
+ * (or a negative SV_E* code) and writes, for the first min(L, max_launches) launches s:
+ *   gates[s]        the number of fused gates the launch applies;
+ *   on_small[s]     1 when it runs on sv_init_apply's small state;
+ *   tile_qubits[s]  0: one gate on a kernel of its own; else a pass, and the local qubits of its tiles
+ *                   (of the small state, numbered by rank, when on_small);
+ *   block_at[s]     the byte offset of the pass's block (and its end at block_at[L] if L < max_launches),
+ * order[0 .. count(f)) = the fused gates' indices in the order they are applied, and each pass's
+ * block that fits blocks_bytes: 168 bytes of geometry (int tile block bits, int[7] their places among
+ * the state's block-index bits, int64[16] float offsets of every eighth tile block, int gates, int
+ * 16-byte units that follow), then the 64-byte gate descriptors and the matrices as the kernel
+ * reads them.  Any output may be NULL. */
+SV_API int sv_fused_plan_passes(const sv_fused *f, int from_basis, int max_launches, int *gates, int *on_small, uint64_t *tile_qubits,
+                                size_t *block_at, int *order, void *blocks, size_t blocks_bytes);
+
 /* ---------------------------------------------------------------------------------------------
  * Learned fusion cost model (no counterpart in the paper's code: the paper tunes its fusion size
  * per machine with a synthetic benchmark, section VI-C; here the simulator learns a cost model

@@ -109,6 +109,7 @@ def _load():
         "sv_fused_get_matrix": (I, [P, I, ctypes.POINTER(ctypes.c_double)]),
         "sv_fused_get_post_phases": (I, [P, I, I, P, P, P]),
         "sv_fused_get_swaps": (I, [P, I, I, P, P]),
+        "sv_fused_plan_passes": (I, [P, I, I, P, P, P, P, P, P, ctypes.c_size_t]),
         "sv_apply_fused_gates": (I, [P, P, ctypes.POINTER(sv_timing)]),
         "sv_init_apply": (I, [P, ctypes.c_uint64, P, ctypes.POINTER(sv_timing)]),
         "sv_norm": (I, [P, ctypes.POINTER(ctypes.c_double)]),
@@ -342,6 +343,33 @@ def sv_apply_fused_gates(h, f, timings: bool = False):
 
 
 # --------------------------------------------------------------------------------------- reductions
+def sv_fused_plan_passes(f, from_basis: bool = False) -> list:
+    """The launches of a call without timing records (host only): per launch its fused gates, whether
+    it runs on sv_init_apply's small state, its tile's local qubits (0: one gate on its own kernel)
+    and the pass's geometry, descriptors and matrices as bytes."""
+    count = sv_fused_count(f)
+    lb = int(bool(from_basis))
+    k = lib.sv_fused_plan_passes(f, lb, 0, None, None, None, None, None, None, 0)
+    if k < 0:
+        _check(k)
+    gates, small = (ctypes.c_int * (k + 1))(), (ctypes.c_int * (k + 1))()
+    tile, at = (ctypes.c_uint64 * (k + 1))(), (ctypes.c_size_t * (k + 1))()
+    order = (ctypes.c_int * max(count, 1))()
+    rc = lib.sv_fused_plan_passes(f, lb, k + 1, gates, small, tile, at, order, None, 0)
+    if rc < 0:
+        _check(rc)
+    blocks = ctypes.create_string_buffer(max(at[k], 1))
+    rc = lib.sv_fused_plan_passes(f, lb, 0, None, None, None, None, None, blocks, at[k])
+    if rc < 0:
+        _check(rc)
+    out, o = [], 0
+    for s in range(k):
+        out.append({"gates": list(order[o:o + gates[s]]), "on_small": bool(small[s]), "tile": int(tile[s]),
+                    "block": blocks.raw[at[s]:at[s + 1]]})
+        o += gates[s]
+    return out
+
+
 def sv_norm(h) -> float:
     out = ctypes.c_double()
     _check(lib.sv_norm(h, ctypes.byref(out)))

@@ -844,36 +844,72 @@ FusedGate remap_gate(const FusedGate &g, uint64_t A, int a)
     return r;
 }
 
-// The launch plan of f's gates (complex64, no timing records): the small-state gates of `lazy` on
-// A's qubits, then the others, each cut into passes and single launches; the passes' descriptors and
-// matrices go to one device buffer.  Made on the first call of each kind and kept with f (its gates,
-// their order and the small-state set never change).
-int ensure_plan(sv_fused *f, sv_fused::Plan *pl, const std::vector<char> *lazy, uint64_t A, int a, int device)
+// The gates that sv_init_apply runs on its small state (one flag per gate) and the qubits A that they
+// name, in one pass over the circuit: a gate qualifies if no earlier gate left out shares a qubit with
+// it (so it commutes past those) and the qubits named so far, its own included, stay within the
+// limit: the light-cone part the fuser placed first (its qubit count), else the default.
+// Returns how many qualify.
+size_t small_state_gates(const sv_fused *f, std::vector<char> *lazy, uint64_t *A)
 {
-    if (pl->ready) return SV_OK;
-    std::vector<const FusedGate *> small, rest;
-    pl->small_gates.clear();
-    pl->small_index.clear();
-    pl->rest_index.clear();
+    const int limit = std::min(f->lazy_limit > 0 ? std::min(f->lazy_limit, kCompactMaxQubits) : kDefaultLazyQubits, f->n - 1);
+    lazy->assign(f->gates.size(), 0);
+    *A = 0;
+    uint64_t blocked = 0;
+    size_t m = 0;
     for (size_t i = 0; i < f->gates.size(); ++i) {
-        if (lazy && (*lazy)[i]) {
-            pl->small_gates.push_back(remap_gate(f->gates[i], A, a));
-            pl->small_index.push_back((int)i);
+        const FusedGate &g = f->gates[i];
+        // a gate with post-phases runs on the full state, and its phases name qubits outside
+        // it: a later gate on those cannot move ahead of it either; so does a swap network
+        uint64_t q = g.mask | g.cmask;
+        for (const FusedGate::PostTerm &t : g.post) q |= uint64_t(1) << t.q;
+        if (!(q & blocked) && __builtin_popcountll(*A | q) <= limit && g.post.empty() && g.swaps.empty()) {
+            *A |= q;
+            (*lazy)[i] = 1;
+            ++m;
         } else {
-            pl->rest_index.push_back((int)i);
-            rest.push_back(&f->gates[i]);
+            blocked |= q;
         }
     }
-    for (const FusedGate &g : pl->small_gates) small.push_back(&g);
-    bool keep_order = false;   // by the circuit's own paths: neither part may be reordered ahead of the other's tensor-core gates
-    for (const FusedGate &g : f->gates) keep_order |= g.path == SV_PATH_TC_TF32 || g.path == SV_PATH_TC_BF16X3;
+    return m;
+}
+
+// The launch plan of f's gates (complex64, no timing records): the small-state gates of `lazy` on
+// A's qubits, then the others, each cut into passes and single launches.  Host only.
+int make_plan(const sv_fused *f, sv_fused::Plan *pl, const std::vector<char> *lazy, uint64_t A, int a)
+{
     try {
+        std::vector<const FusedGate *> small, rest;
+        pl->small_gates.clear();
+        pl->small_index.clear();
+        pl->rest_index.clear();
+        bool keep_order = false;   // by the circuit's own paths: neither part may be reordered ahead of the other's tensor-core gates
+        for (size_t i = 0; i < f->gates.size(); ++i) {
+            const FusedGate &g = f->gates[i];
+            keep_order |= g.path == SV_PATH_TC_TF32 || g.path == SV_PATH_TC_BF16X3;
+            if (lazy && (*lazy)[i]) {
+                pl->small_gates.push_back(remap_gate(g, A, a));
+                pl->small_index.push_back((int)i);
+            } else {
+                pl->rest_index.push_back((int)i);
+                rest.push_back(&g);
+            }
+        }
+        for (const FusedGate &g : pl->small_gates) small.push_back(&g);
         plan_passes(small, a, keep_order, &pl->small);
         plan_passes(rest, f->n, keep_order, &pl->rest);
     } catch (const std::exception &) {
         set_error("sv_apply_fused_gates: out of host memory for the launch plan");
         return SV_ENOMEM;
     }
+    return SV_OK;
+}
+
+// The plan of a call, its passes' descriptors and matrices in one device buffer.  Made on the first
+// call of each kind and kept with f (its gates, their order and the small-state set never change).
+int ensure_plan(sv_fused *f, sv_fused::Plan *pl, const std::vector<char> *lazy, uint64_t A, int a, int device)
+{
+    if (pl->ready) return SV_OK;
+    SV_TRY(make_plan(f, pl, lazy, A, a));
     const size_t ns = pl->small.image.size(), nr = pl->rest.image.size();
     pl->rest_off = ns;
     const size_t bytes = (ns + nr) * sizeof(float);
@@ -1097,34 +1133,56 @@ extern "C" int sv_init_apply(sv_state *st, uint64_t basis_index, const sv_fused 
     sv_fused *f = const_cast<sv_fused *>(fc);
     if (f->n != st->n) { set_error("sv_init_apply: circuit is for %d qubits, state has %d", f->n, st->n); return SV_ESTATE; }
     if (basis_index >> st->n) { set_error("sv_init_apply: basis index out of range for %d qubits", st->n); return SV_EINVAL; }
-    // gates for the small state, in one pass over the circuit: a gate qualifies if no earlier gate
-    // left out shares a qubit with it (so it commutes past those) and the qubits named so far, its
-    // own included, stay within the limit
-    // the light-cone part the fuser placed first (its qubit count), else the default
-    const int limit = std::min(f->lazy_limit > 0 ? std::min(f->lazy_limit, kCompactMaxQubits) : kDefaultLazyQubits, st->n - 1);
-    std::vector<char> lazy(f->gates.size(), 0);
-    uint64_t A = 0, blocked = 0;
-    size_t m = 0;
-    if (!st->c128)
-        for (size_t i = 0; i < f->gates.size(); ++i) {
-            const FusedGate &g = f->gates[i];
-            // a gate with post-phases runs on the full state, and its phases name qubits outside
-            // it: a later gate on those cannot move ahead of it either; so does a swap network
-            uint64_t q = g.mask | g.cmask;
-            for (const FusedGate::PostTerm &t : g.post) q |= uint64_t(1) << t.q;
-            if (!(q & blocked) && __builtin_popcountll(A | q) <= limit && g.post.empty() && g.swaps.empty()) {
-                A |= q;
-                lazy[i] = 1;
-                ++m;
-            } else {
-                blocked |= q;
-            }
-        }
+    std::vector<char> lazy;
+    uint64_t A = 0;
+    const size_t m = st->c128 ? 0 : small_state_gates(f, &lazy, &A);
     if (m == 0) {
         SV_TRY(sv_init(st, basis_index));
         return apply_core(st, f, timings, nullptr, 0, 0, "sv_init_apply");
     }
     return apply_core(st, f, timings, &lazy, A, basis_index, "sv_init_apply");
+}
+
+extern "C" int sv_fused_plan_passes(const sv_fused *f, int from_basis, int max_launches, int *gates, int *on_small, uint64_t *tile_qubits,
+                                    size_t *block_at, int *order, void *blocks, size_t blocks_bytes)
+{
+    clear_error();
+    if (!f || max_launches < 0) { set_error("sv_fused_plan_passes: bad argument"); return SV_EINVAL; }
+    sv_fused::Plan pl;
+    int launches = 0;
+    try {
+        std::vector<char> lazy;
+        uint64_t A = 0;
+        const size_t m = from_basis ? small_state_gates(f, &lazy, &A) : 0;
+        SV_TRY(make_plan(f, &pl, m > 0 ? &lazy : nullptr, m > 0 ? A : 0, m > 0 ? __builtin_popcountll(A) : 0));
+        size_t at = 0, o = 0;
+        for (int part = 0; part < 2; ++part) {
+            const PassPlan &p = part ? pl.rest : pl.small;
+            const std::vector<int> &index = part ? pl.rest_index : pl.small_index;
+            for (const PassStep &s : p.steps) {
+                std::vector<unsigned char> block;
+                if (s.single < 0) pass_block(p, s, &block);
+                if (blocks && at + block.size() <= blocks_bytes) std::memcpy(static_cast<unsigned char *>(blocks) + at, block.data(), block.size());
+                if (launches < max_launches) {
+                    if (gates) gates[launches] = s.single < 0 ? (int)s.gates.size() : 1;
+                    if (on_small) on_small[launches] = part == 0;
+                    if (tile_qubits) tile_qubits[launches] = s.tile;
+                    if (block_at) block_at[launches] = at;
+                }
+                at += block.size();
+                if (order) {
+                    if (s.single < 0) for (int g : s.gates) order[o++] = index[(size_t)g];
+                    else order[o++] = index[(size_t)s.single];
+                }
+                ++launches;
+            }
+        }
+        if (block_at && launches < max_launches) block_at[launches] = at;
+    } catch (const std::exception &) {
+        set_error("sv_fused_plan_passes: out of host memory");
+        return SV_ENOMEM;
+    }
+    return launches;
 }
 
 extern "C" int sv_device_status(void)

@@ -130,6 +130,8 @@ struct PassStep {
     int single = -1;
     int kmax = 0;               // largest gate of the pass
     long long tiles = 0;
+    uint64_t tile = 0;          // its local qubits
+    std::vector<int> gates;     // what it applies, in order (indices into the planned gates)
     std::vector<unsigned long long> args;   // the pass's kernel arguments
     size_t image_off = 0;       // its descriptors and matrices: floats into PassPlan::image
 };
@@ -142,6 +144,8 @@ struct PassPlan {
 // gate anywhere keeps its order (the operand split turns a last-bit difference of the input into a
 // larger one).
 void plan_passes(const std::vector<const FusedGate *> &gates, int n, bool keep_order, PassPlan *plan);
+// A pass's geometry, descriptors and matrices as they reach its kernel (sv_fused_plan_passes).
+void pass_block(const PassPlan &plan, const PassStep &p, std::vector<unsigned char> *out);
 int launch_stage(float *sv, const float *image, const PassStep &p, cudaStream_t stream, int num_sms);
 
 // Tensor-core path (sv_tc.cu): host-side operand images and the launcher.

@@ -390,6 +390,8 @@ void plan_passes(const std::vector<const FusedGate *> &gates, int n, bool keep_o
             for (int q = 5; q < n && __builtin_popcountll(lam) < L; ++q) lam |= uint64_t(1) << q;   // whole tiles: lowest free qubits
             for (int t : took) st.kmax = std::max(st.kmax, gates[(size_t)t]->k);
             st.tiles = 1ll << (n - L);
+            st.tile = lam;
+            st.gates = took;
             st.image_off = plan->image.size();
             st.args.assign((sizeof(StageArgs) + 7) / 8, 0);
             fill_stage(gates, took, lam, n, reinterpret_cast<StageArgs *>(st.args.data()), &plan->image);
@@ -397,6 +399,15 @@ void plan_passes(const std::vector<const FusedGate *> &gates, int n, bool keep_o
         plan->steps.push_back(std::move(st));
         left.swap(rest);
     }
+}
+
+void pass_block(const PassPlan &plan, const PassStep &p, std::vector<unsigned char> *out)
+{
+    const StageArgs *a = reinterpret_cast<const StageArgs *>(p.args.data());
+    static_assert(sizeof(StageArgs) == 168, "sv_fused_plan_passes documents the layout");
+    out->resize(sizeof(StageArgs) + 16 * (size_t)a->units);
+    std::memcpy(out->data(), a, sizeof(StageArgs));
+    std::memcpy(out->data() + sizeof(StageArgs), plan.image.data() + p.image_off, 16 * (size_t)a->units);
 }
 
 namespace {
