@@ -2,6 +2,7 @@
 Every address a thread forms lies in its tile (or in the state), the groups of a gate are disjoint
 and complete, tiles are copied whole and once, and a numpy run of the passes gives the oracle's state."""
 import struct
+import time
 
 import numpy as np
 import pytest
@@ -238,4 +239,60 @@ def test_order_is_kept_around_tensor_core_gates(B, from_basis):
     f = B.sv_fuse_circuit(gates, n, mode=B.FUSE_NONE)   # without tensor cores gates do move
     order = [g for s in B.sv_fused_plan_passes(f) for g in s["gates"]]
     assert order != sorted(order)
+    B.sv_fused_free(f)
+
+
+def scan_plan(B, f, n, keep_order):
+    """The passes by scans of all gates left: a gate joins when none left out before it shares a qubit
+    with it and it fits (states below 21 qubits, where every run of two or more is a pass)."""
+    infos = [B.sv_fused_get_info(f, i) for i in range(B.sv_fused_count(f))]
+    masks = [sum(1 << q for q in i["targets"]) for i in infos]
+    named = [m | sum(1 << q for q in i["controls"]) for m, i in zip(masks, infos)]
+    fits = [i["path"] == B.PATH_CONTROLLED or (i["path"] in (B.PATH_LOW, B.PATH_HIGH, B.PATH_MIXED) and i["k"] <= 5) for i in infos]
+    tile = min(n, 12 if n >= 19 else 10 if n <= 16 and max(i["k"] for i in infos) <= 2 else 11)
+    left, out = list(range(len(infos))), []
+    while left:
+        lam, blocked, floats, took, rest = 31, 0, 0, [], []
+        for s, g in enumerate(left):
+            if (fits[g] and not named[g] & blocked and bin(lam | masks[g]).count("1") <= tile and len(took) < 48
+                    and floats + 2 * 4 ** infos[g]["k"] <= 4096):
+                lam |= masks[g]
+                floats += 2 * 4 ** infos[g]["k"]
+                took.append(g)
+                continue
+            if not took:
+                took.append(g)
+                rest += left[s + 1:]
+                break
+            blocked |= named[g]
+            rest.append(g)
+            if keep_order:
+                rest += left[s + 1:]
+                break
+        out.append(took)
+        left = rest
+    return out
+
+
+@pytest.mark.parametrize("n", [6, 13, 17, 20])
+@pytest.mark.parametrize("max_k,precision", [(1, 0), (2, 0), (4, 0), (6, 0), (6, 2)])
+def test_plan_is_the_first_fit_by_scans(B, n, max_k, precision):
+    gates = circuit(n, min(max_k, 3), seed=n * max_k, count=150)
+    f = B.sv_fuse_circuit(gates, n, max_k=min(max_k, n), precision=precision, tc_min_k=4)
+    paths = {B.sv_fused_get_info(f, i)["path"] for i in range(B.sv_fused_count(f))}
+    want = scan_plan(B, f, n, bool(paths & {B.PATH_TC_TF32, B.PATH_TC_BF16X3}))
+    assert [s["gates"] for s in B.sv_fused_plan_passes(f)] == want
+    B.sv_fused_free(f)
+
+
+def test_planning_time_grows_with_the_gates(B):
+    """200,000 unfused gates: 0.26 s with their images; scans of all gates left took 21 s."""
+    n, rng = 20, np.random.default_rng(0)
+    u = [wl.random_unitary(4, rng) for _ in range(8)]
+    pairs = rng.integers(0, n, (200000, 2))
+    gates = [wl.Gate((int(a), int(b)), u[i % 8], (), "g") for i, (a, b) in enumerate(pairs) if a != b]
+    f = B.sv_fuse_circuit(gates, n, mode=B.FUSE_NONE)
+    began = time.monotonic()
+    assert B.lib.sv_fused_plan_passes(f, 0, 0, None, None, None, None, None, None, 0) > 1000
+    assert time.monotonic() - began < 5.0
     B.sv_fused_free(f)
