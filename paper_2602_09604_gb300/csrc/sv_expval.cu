@@ -29,9 +29,11 @@
 // accumulator.
 #include <algorithm>
 #include <cstring>
+#include <exception>
 #include <mutex>
 #include <vector>
 
+#include "sv_evplan.h"
 #include "sv_internal.h"
 #include "sv_tile.h"
 
@@ -406,10 +408,6 @@ constexpr int kEvtSmem = (8 << kEvtQubits) + 16 * kEvtThreads * (int)sizeof(floa
 
 // The tile pass of the strings order[..] listed in `runs` (each a run of equal x masks); res[i]
 // receives the i-th string's sum in the order of `placed`.
-struct EvRun {
-    int pos, m;   // order[pos .. pos + m)
-};
-
 void fill_tiles(const std::vector<EvRun> &runs, const std::vector<int> &order, const uint64_t *x_masks, const uint64_t *z_masks, int n,
                 uint64_t lam, EvtArgs *a, std::vector<int> *placed)
 {
@@ -501,9 +499,10 @@ int highest_bit(unsigned long long v)
 
 using namespace svg;
 
-extern "C" int sv_expval_pauli(const sv_state *st_c, const uint64_t *x_masks, const uint64_t *z_masks, int count, double *out)
+namespace {
+
+int expval_pauli(const sv_state *st_c, const uint64_t *x_masks, const uint64_t *z_masks, int count, double *out)
 {
-    clear_error();
     sv_state *st = const_cast<sv_state *>(st_c);
     if (!st || count < 0 || (count > 0 && (!x_masks || !z_masks || !out))) { set_error("sv_expval_pauli: bad argument"); return SV_EINVAL; }
     if (st->c128) { set_error("sv_expval_pauli: expectation values need a complex64 state"); return SV_EINVAL; }
@@ -544,44 +543,24 @@ extern "C" int sv_expval_pauli(const sv_state *st_c, const uint64_t *x_masks, co
     // qubits share a read of the state; a tile pass is taken when it replaces two or more passes of the
     // kernel above (its own work per string is larger, so one pass alone is better left there).
     std::vector<EvRun> runs, left;
+    std::vector<uint64_t> run_x;
     for (int p = 0; p < count;) {
+        const uint64_t x = x_masks[order[(size_t)p]];
         int m = 0;
-        while (p + m < count && m < kEvtStrings / 2 && x_masks[order[(size_t)(p + m)]] == x_masks[order[(size_t)p]]) ++m;
+        while (p + m < count && m < kEvtStrings / 2 && x_masks[order[(size_t)(p + m)]] == x) ++m;
         runs.push_back(EvRun{p, m});
+        run_x.push_back(x);
         p += m;
     }
     if (n >= kEvtMinQubits) {
-        while (!runs.empty()) {
-            uint64_t lam = 31;
-            int strings = 0, passes = 0;
-            std::vector<EvRun> took, rest;
-            for (const EvRun &r : runs) {
-                const uint64_t with = lam | x_masks[order[(size_t)r.pos]];
-                if (__builtin_popcountll(with) <= kEvtQubits && strings + r.m <= kEvtStrings && 2 * (took.size() + 1) <= kEvtGroups) {
-                    lam = with;
-                    strings += r.m;
-                    passes += (r.m + kEvMaxStrings - 1) / kEvMaxStrings;
-                    took.push_back(r);
-                } else {
-                    rest.push_back(r);
-                }
-            }
-            if (took.empty()) {   // the first run's mask fits no tile
-                left.push_back(runs.front());
-                runs.erase(runs.begin());
-                continue;
-            }
-            if (passes < 2) {
-                left.insert(left.end(), took.begin(), took.end());
-            } else {
-                for (int q = 5; q < n && __builtin_popcountll(lam) < kEvtQubits; ++q) lam |= uint64_t(1) << q;
-                EvtArgs a;
-                std::vector<int> placed;
-                fill_tiles(took, order, x_masks, z_masks, n, lam, &a, &placed);
-                SV_TRY(launch_tiles(st->d, a, partials, results + out_pos, st->num_sms, st->stream));
-                for (int s : placed) slot_of[(size_t)s] = out_pos++;
-            }
-            runs.swap(rest);
+        std::vector<EvTilePass> tiles;
+        plan_tiles(runs, run_x, n, EvTileLimits{kEvtQubits, kEvtStrings, kEvtGroups, 2, kEvMaxStrings}, &tiles, &left);
+        for (const EvTilePass &t : tiles) {
+            EvtArgs a;
+            std::vector<int> placed;
+            fill_tiles(t.runs, order, x_masks, z_masks, n, t.lam, &a, &placed);
+            SV_TRY(launch_tiles(st->d, a, partials, results + out_pos, st->num_sms, st->stream));
+            for (int s : placed) slot_of[(size_t)s] = out_pos++;
         }
     } else {
         left.swap(runs);
@@ -642,4 +621,17 @@ extern "C" int sv_expval_pauli(const sv_state *st_c, const uint64_t *x_masks, co
         }
     }
     return SV_OK;
+}
+
+}  // namespace
+
+extern "C" int sv_expval_pauli(const sv_state *st, const uint64_t *x_masks, const uint64_t *z_masks, int count, double *out)
+{
+    clear_error();
+    try {
+        return expval_pauli(st, x_masks, z_masks, count, out);
+    } catch (const std::exception &) {   // the vectors of many strings
+        set_error("sv_expval_pauli: out of host memory");
+        return SV_ENOMEM;
+    }
 }
