@@ -244,8 +244,9 @@ SV_API int sv_fused_get_matrix(const sv_fused *f, int i, double *out);
  * given fused circuit uploads the matrices that do not travel as kernel arguments (k = 6 and the
  * tensor-core operands) with cudaMalloc/cudaMemcpy.  Without `timings`, CUDA-core fp32 gates whose
  * qubits lie close together share passes over the state (a gate only moves ahead of gates on other
- * qubits; the plan and its matrices are made and uploaded on the first such call, and a call on a
- * stream that is being captured before that launches gate by gate).  With `timings` non-NULL (one
+ * qubits; the plan and its matrices are made and uploaded on the first such call, without waiting for
+ * work queued on any stream, and a call on a stream that is being captured before that launches gate by
+ * gate).  With `timings` non-NULL (one
  * record per fused gate) every gate has its own launch, bracketed by CUDA events, and the call
  * synchronises.
  *

@@ -905,7 +905,7 @@ int make_plan(const sv_fused *f, sv_fused::Plan *pl, const std::vector<char> *la
 }
 
 // The plan of a call, its passes' descriptors and matrices in one device buffer.  Made on the first
-// call of each kind and kept with f (its gates, their order and the small-state set never change).
+// call of each kind, which waits for this upload but for no work queued on any stream, and kept with f (its gates, their order and the small-state set never change).
 int ensure_plan(sv_fused *f, sv_fused::Plan *pl, const std::vector<char> *lazy, uint64_t A, int a, int device)
 {
     if (pl->ready) return SV_OK;
@@ -914,6 +914,7 @@ int ensure_plan(sv_fused *f, sv_fused::Plan *pl, const std::vector<char> *lazy, 
     pl->rest_off = ns;
     const size_t bytes = (ns + nr) * sizeof(float);
     if (bytes > 0) {
+        const RelaxedCapture relaxed;
         SharedBuffer *buf = nullptr;
         SV_TRY(shared_buffer_get(device, bytes, &buf));
         std::unique_lock<std::mutex> lk;
@@ -922,11 +923,7 @@ int ensure_plan(sv_fused *f, sv_fused::Plan *pl, const std::vector<char> *lazy, 
         if (rc == SV_OK) {
             if (ns) std::memcpy(img, pl->small.image.data(), ns * sizeof(float));
             if (nr) std::memcpy(img + ns * sizeof(float), pl->rest.image.data(), nr * sizeof(float));
-            const cudaError_t e = cudaMemcpy(buf->p, img, bytes, cudaMemcpyHostToDevice);
-            if (e != cudaSuccess) {
-                set_error("sv_apply_fused_gates: pass images: %s", cudaGetErrorString(e));
-                rc = SV_ECUDA;
-            }
+            rc = upload_now(device, buf->p, img, bytes);
         }
         if (rc != SV_OK) {
             shared_buffer_release(buf);
@@ -1216,7 +1213,7 @@ extern "C" void sv_fused_free(sv_fused *f)
         dev_buffer_put(f->device, f->d_buf, f->d_buf_bytes);
         dev_buffer_put(f->device, f->d_mats64, f->d_mats64_bytes);
         for (sv_fused::Plan &p : f->plans) shared_buffer_release(p.buf);
-        shared_buffers_collect();
+        shared_buffers_collect(true);
         if (f->device >= 0 && cur >= 0 && cur != f->device) cudaSetDevice(cur);
     }
     delete f;

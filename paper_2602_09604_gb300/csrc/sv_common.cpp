@@ -52,21 +52,6 @@ void shared_buffer_release(SharedBuffer *b)
     g_dropped = b;
 }
 
-void shared_buffers_collect()
-{
-    SharedBuffer *b = nullptr;
-    {
-        std::lock_guard<std::mutex> lk(g_buf_mu);
-        std::swap(b, g_dropped);
-    }
-    while (b) {
-        SharedBuffer *next = b->next;
-        dev_buffer_put(b->device, b->p, b->bytes);
-        delete b;
-        b = next;
-    }
-}
-
 int shared_buffer_retain_in_capture(SharedBuffer *b, cudaStream_t stream)
 {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
@@ -89,7 +74,7 @@ int dev_buffer_get(int device, size_t bytes, void **out, size_t *got_bytes)
 {
     *out = nullptr;
     *got_bytes = 0;
-    shared_buffers_collect();
+    shared_buffers_collect(false);
     if (device >= 0 && device < 64) {
         std::lock_guard<std::mutex> lk(g_buf_mu);
         std::vector<DevBuf> &c = g_buf_cache[device];
@@ -108,24 +93,63 @@ int dev_buffer_get(int device, size_t bytes, void **out, size_t *got_bytes)
     return SV_OK;
 }
 
+namespace {
+// whether the cache took the buffer
+bool cache_buffer(int device, void *p, size_t bytes)
+{
+    if (device < 0 || device >= 64) return false;
+    std::lock_guard<std::mutex> lk(g_buf_mu);
+    std::vector<DevBuf> &c = g_buf_cache[device];
+    size_t held = 0;
+    for (const DevBuf &b : c) held += b.bytes;
+    if (c.size() >= kBufCacheCount || held + bytes > kBufCacheBytes) return false;
+    c.push_back(DevBuf{p, bytes});
+    return true;
+}
+}  // namespace
+
 void dev_buffer_put(int device, void *p, size_t bytes)
 {
-    if (!p) return;
-    if (device >= 0 && device < 64) {
-        std::lock_guard<std::mutex> lk(g_buf_mu);
-        std::vector<DevBuf> &c = g_buf_cache[device];
-        size_t held = 0;
-        for (const DevBuf &b : c) held += b.bytes;
-        if (c.size() < kBufCacheCount && held + bytes <= kBufCacheBytes) {
-            c.push_back(DevBuf{p, bytes});
-            return;
-        }
-    }
+    if (!p || cache_buffer(device, p, bytes)) return;
     int cur = -1;
     cudaGetDevice(&cur);
     if (device >= 0 && cur != device) cudaSetDevice(device);
     cudaFree(p);
     if (device >= 0 && cur >= 0 && cur != device) cudaSetDevice(cur);
+}
+
+void shared_buffers_collect(bool may_free)
+{
+    SharedBuffer *b = nullptr;
+    {
+        std::lock_guard<std::mutex> lk(g_buf_mu);
+        std::swap(b, g_dropped);
+    }
+    while (b) {
+        SharedBuffer *next = b->next;
+        if (may_free) dev_buffer_put(b->device, b->p, b->bytes);
+        if (may_free || cache_buffer(b->device, b->p, b->bytes)) {
+            delete b;
+        } else {
+            std::lock_guard<std::mutex> lk(g_buf_mu);
+            b->next = g_dropped;
+            g_dropped = b;
+        }
+        b = next;
+    }
+}
+
+int upload_now(int device, void *dst, const void *pinned, size_t bytes)
+{
+    static std::mutex mu;
+    static cudaStream_t streams[64] = {};
+    if (device < 0 || device >= 64) { set_error("upload: device %d out of range", device); return SV_EINVAL; }
+    std::lock_guard<std::mutex> lk(mu);
+    cudaStream_t &s = streams[device];
+    if (!s) SV_CUDA_TRY(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+    SV_CUDA_TRY(cudaMemcpyAsync(dst, pinned, bytes, cudaMemcpyHostToDevice, s));
+    SV_CUDA_TRY(cudaStreamSynchronize(s));
+    return SV_OK;
 }
 
 namespace {

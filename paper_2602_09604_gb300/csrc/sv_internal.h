@@ -166,8 +166,8 @@ void dev_buffer_put(int device, void *p, size_t bytes);
 // A buffer of that cache with more than one owner: a fused circuit's pass images belong to the
 // circuit and to every graph captured from it, so a graph can be replayed after the circuit is
 // freed.  The last release puts it aside without a CUDA call (a graph's end may be reported where
-// none is allowed); shared_buffers_collect, called by dev_buffer_get too, puts such buffers back into
-// the cache.
+// none is allowed); shared_buffers_collect puts such buffers back into the cache and, with may_free,
+// frees what the cache does not keep (cudaFree waits for the device: dev_buffer_get collects without).
 struct SharedBuffer {
     std::atomic<int> owners{1};
     int device = -1;
@@ -177,7 +177,17 @@ struct SharedBuffer {
 };
 int shared_buffer_get(int device, size_t bytes, SharedBuffer **out);
 void shared_buffer_release(SharedBuffer *b);
-void shared_buffers_collect();
+void shared_buffers_collect(bool may_free);
+// Copies pinned memory to the device on a stream of the library's own and waits for that copy alone:
+// not for work queued on the legacy stream, as cudaMemcpy does.
+int upload_now(int device, void *dst, const void *pinned, size_t bytes);
+// While it lives, calls on this thread that CUDA refuses during another stream's capture (allocations,
+// waits) are allowed and leave that capture valid.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
 // Makes the graph that `stream` is being captured into an owner (and with it every executable graph
 // made from it, until its last replay has ended).
 int shared_buffer_retain_in_capture(SharedBuffer *b, cudaStream_t stream);
