@@ -247,7 +247,12 @@ bool stageable(const FusedGate &g)
 
 // Time of a gate on its own kernel, and its share in a pass, on states past the L2 in units of one read
 // and write of the state at the copy rate (k = 1..5; 28 qubits: 1.0 = 0.63 ms).  A pass adds
-// kPassCost for its own read and write, partly hidden behind the arithmetic.
+// kPassCost for its own read and write, partly hidden behind the arithmetic.  Below 28 qubits the same
+// figures serve as a rule; measured by it / every pass taken / every gate alone (us, grids of 10
+// cycles, gates of 4): 21 qubits 161 / 166 / 185, 23 qubits 567 / 616 / 633, 24 qubits 1229 / 1220 / 1414,
+// 26 qubits 5518 / 5572 / 6101.  It loses most, 2 to 3%, on quantum volume with gates of 4 (24 qubits
+// 868 / 843 / 980, 26 qubits 3484 / 3400 / 3672), and below 21 qubits it costs up to a third (19 qubits
+// 48 / 35 / 83): there every pass is taken.
 constexpr double kPassCost = 0.7, kInPass[6] = {0, 0.2, 0.3, 0.5, 1.0, 2.0};
 double alone_cost(const FusedGate &g)
 {
@@ -357,10 +362,11 @@ void plan_passes(const std::vector<const FusedGate *> &gates, int n, bool keep_o
         }
     }
     // Large tiles hold more gates a pass; on a small state they leave SMs without a tile, and a pass is
-    // then as long as its chain of gates on one tile.  Measured (us, tiles of 2^10 / 2^11 / 2^12):
-    // 16 qubits, gates of 2: 68 / 79 / 103, of 4: 86 / 65 / 67; 18 qubits, 2: 82 / 62 / 78;
-    // 19 qubits, 3: 139 / 94 / 72; 22 qubits, 4: 573 / 464 / 278.
-    const int L = std::min(n, n >= 19 ? kStageQubits : n <= 16 && small ? kStageQubits - 2 : kStageQubits - 1);
+    // then as long as its chain of gates on one tile.  Measured (us, tiles of 2^10 / 2^11 / 2^12; grids of
+    // 14 cycles): gates of 2, 16 qubits 47 / 59 / 85, 17 qubits 46 / 60 / 85, 18 qubits 98 / 73 / 98;
+    // gates of 4, 16 qubits 61 / 43 / 47, 17 qubits 42 / 42 / 64; gates of 3, 18 qubits 83 / 57 / 77,
+    // 19 qubits 204 / 128 / 88, 20 qubits 380 / 226 / 190.
+    const int L = std::min(n, n >= 19 ? kStageQubits : n <= 17 && small ? kStageQubits - 2 : kStageQubits - 1);
     std::vector<int> took, held;
     while (!ready.empty()) {
         PassStep st;

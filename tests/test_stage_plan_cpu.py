@@ -249,7 +249,7 @@ def scan_plan(B, f, n, keep_order):
     masks = [sum(1 << q for q in i["targets"]) for i in infos]
     named = [m | sum(1 << q for q in i["controls"]) for m, i in zip(masks, infos)]
     fits = [i["path"] == B.PATH_CONTROLLED or (i["path"] in (B.PATH_LOW, B.PATH_HIGH, B.PATH_MIXED) and i["k"] <= 5) for i in infos]
-    tile = min(n, 12 if n >= 19 else 10 if n <= 16 and max(i["k"] for i in infos) <= 2 else 11)
+    tile = min(n, 12 if n >= 19 else 10 if n <= 17 and max(i["k"] for i in infos) <= 2 else 11)
     left, out = list(range(len(infos))), []
     while left:
         lam, blocked, floats, took, rest = 31, 0, 0, [], []
