@@ -368,10 +368,13 @@ SV_API int sv_alloc_c128(int n_qubits, void *dev_ptr, size_t bytes, void *cuda_s
  *     sigma_q = X if bit q is set in x_masks[p] only, Z if in z_masks[p] only, Y if in both, else I,
  * and out[p] (host array of count doubles) = <psi|P_p|psi>, real because P_p is Hermitian; the
  * state is not normalised first (divide by sv_norm for a state that is not unit-norm).  Each
- * amplitude's term is formed in fp32 and accumulated in float-float per thread, fp64 across
- * threads, in a fixed order (deterministic).  Strings sharing an x mask share read passes, up to 8
- * strings per pass over the 8 * 2^n bytes; on states of 26 or more qubits strings with different x masks
- * share passes too (up to 64 strings whose x masks touch at most 7 qubits above qubit 4).  SV_EINVAL if a mask has a bit >= n.  Grows a small
+ * amplitude's term is formed in fp32, eight (pairs of) terms are summed in fp32, these sums in
+ * float-float per thread and fp64 across threads, in a fixed order (deterministic).  A string's error is
+ * at most 18 * 2^-24 of the sum over j of |c_(j^x)| |c_j| (<= 1 for a unit state); on states without
+ * structure roundings cancel and it is orders of magnitude smaller.  Strings sharing an x mask share
+ * read passes, up to 8 strings per pass over the 8 * 2^n bytes; on states of 26 or more qubits
+ * strings with different x masks share passes too (up to 64 strings whose x masks touch at most 7 qubits
+ * above qubit 4), with sums in another order.  SV_EINVAL if a mask has a bit >= n.  Grows a small
  * workspace on the state's device when count exceeds the previous maximum.  Synchronises. */
 SV_API int sv_expval_pauli(const sv_state *st, const uint64_t *x_masks, const uint64_t *z_masks, int count, double *out);
 

@@ -292,8 +292,20 @@ int launch_ev(const float *sv, const EvArgs &a, double *partials, unsigned *coun
 // name any qubit.  Terms of a pair (j, j ^ x) are equal once signed, so only one of each pair is formed.
 constexpr int kEvtThreads = 128;
 constexpr int kEvtQubits = 12;
-// From here on the two kernels' sums agree to 1e-9 (the rounding of the fp32 terms' sums averages out
-// with the number of terms: 4e-9 apart at 20 qubits); smaller states keep the one-mask kernel's sums.
+constexpr int kEvtTileFloats = 2 << kEvtQubits;
+// Tile passes start here although they are faster from 12 qubits on and no less exact: values are
+// returned in 64 bits, the two kernels round in other places, and below this size what they
+// return differs by more than 1e-9 even on states without structure (relative 2-norm over a chain's
+// strings, random amplitudes on a product state; one-mask / tile time of the XYZ chain, and the largest
+// difference of the XYZ and X-ZZ chains):
+//     20 qubits   345 /  103 us   6e-9        25 qubits  1781 /  639 us   2e-9
+//     23 qubits   725 /  235 us   2e-9        26 qubits  3283 / 1287 us   6e-10
+//     24 qubits  1099 /  370 us   2e-9        27 qubits  6359 / 2520 us   6e-10
+// On states whose terms repeat in a pattern both are off by up to 1e-7 at every size.  The bound of a
+// string's error is 5 * 2^-24 of the sum of |c_(j^x)| |c_j| (two roundings a term, three levels of
+// sums); the one-mask kernel's is 6 * 2^-24 with four or more strings a pass and up to 18 * 2^-24 with
+// fewer.  Measured against 64 bits on the states above: 20 qubits 1.8e-9 (one-mask) and 1.2e-9
+// (tiles), 24 qubits 5.9e-10 and 3.1e-10, 26 qubits 2.4e-10 and 2.0e-10.
 constexpr int kEvtMinQubits = 26;
 constexpr int kEvtCtas = 4;      // per SM: 53 KB of shared memory, 128 registers a thread
 constexpr int kEvtGroups = 32;
@@ -325,7 +337,7 @@ __global__ void __launch_bounds__(kEvtThreads, kEvtCtas) expval_tile_kernel(cons
 {
     extern __shared__ __align__(16) float smem[];
     float *tile = smem;
-    float *rb = smem + (64 << a.t.fb);                              // 16 x 128 entries
+    float *rb = smem + kEvtTileFloats;                              // 16 x 128 entries
     float2 *acc = reinterpret_cast<float2 *>(rb + 16 * kEvtThreads);   // per string and lane
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const TileMover<kEvtThreads> mv(a.t);
@@ -404,7 +416,7 @@ __global__ void __launch_bounds__(128) expval_sum_kernel(const double *__restric
     if (threadIdx.x == 0) result[blockIdx.x] = (red[0] + red[1]) + (red[2] + red[3]);
 }
 
-constexpr int kEvtSmem = (8 << kEvtQubits) + 16 * kEvtThreads * (int)sizeof(float) + kEvtStrings * 32 * (int)sizeof(float2);
+constexpr int kEvtSmem = (int)sizeof(float) * (kEvtTileFloats + 16 * kEvtThreads) + kEvtStrings * 32 * (int)sizeof(float2);
 
 // The tile pass of the strings order[..] listed in `runs` (each a run of equal x masks); res[i]
 // receives the i-th string's sum in the order of `placed`.
@@ -476,7 +488,7 @@ int launch_tiles(const float *sv, const EvtArgs &a, double *partials, double *re
         }
     }
     const int grid = (int)std::min<long long>(a.tiles, (long long)kEvtCtas * num_sms);
-    const int smem = (int)sizeof(float) * (64 << a.t.fb) + 16 * kEvtThreads * (int)sizeof(float) + a.n_strings * 32 * (int)sizeof(float2);
+    const int smem = (int)sizeof(float) * (kEvtTileFloats + 16 * kEvtThreads) + a.n_strings * 32 * (int)sizeof(float2);
     expval_tile_kernel<<<grid, kEvtThreads, smem, s>>>(sv, a, partials);
     SV_CUDA_TRY(cudaGetLastError());
     expval_sum_kernel<<<a.n_strings, 128, 0, s>>>(partials, grid, a.n_strings, result);
@@ -541,7 +553,8 @@ int expval_pauli(const sv_state *st_c, const uint64_t *x_masks, const uint64_t *
     int out_pos = 0;   // next slot of `results`
     // Runs of equal x masks (cut at half a tile pass's strings).  Runs whose masks fit one tile's local
     // qubits share a read of the state; a tile pass is taken when it replaces two or more passes of the
-    // kernel above (its own work per string is larger, so one pass alone is better left there).
+    // kernel above.  26 qubits, tile / one-mask (us): one string 127 / 110, eight of one mask 152 / 160,
+    // two masks 149 / 192, 16 of one mask 168 / 297, two masks of eight 206 / 298, seven of eight 435 / 959.
     std::vector<EvRun> runs, left;
     std::vector<uint64_t> run_x;
     for (int p = 0; p < count;) {
