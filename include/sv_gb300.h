@@ -244,19 +244,20 @@ SV_API int sv_fused_get_matrix(const sv_fused *f, int i, double *out);
  * given fused circuit uploads the matrices that do not travel as kernel arguments (k = 6 and the
  * tensor-core operands) with cudaMalloc/cudaMemcpy.  Without `timings`, CUDA-core fp32 gates whose
  * qubits lie close together share passes over the state (a gate only moves ahead of gates on other
- * qubits; the plan and its matrices are made and uploaded on the first such call, without waiting for
- * work queued on any stream, and a call on a stream that is being captured before that launches gate by
- * gate).  With `timings` non-NULL (one
- * record per fused gate) every gate has its own launch, bracketed by CUDA events, and the call
- * synchronises.
+ * qubits).  The plan is made on the first such call; its matrices are uploaded by the first call on a
+ * stream not being captured that they pay for (the first, unless the circuit is short and the state
+ * small), without waiting for work queued on any stream.  Calls before that launch gate by gate, in the
+ * same order and with the same bits.  With `timings` non-NULL (one record per fused gate) every gate has
+ * its own launch, in circuit order, bracketed by CUDA events, and the call synchronises.
  *
  * A graph captured from a call (also of sv_init_apply) keeps the shared passes' matrices alive by
  * itself: it may be replayed after sv_fused_free.  Matrices of k = 6 gates and tensor-core operands
  * belong to the fused circuit: a graph with such gates is replayed only while the circuit exists. */
 SV_API int sv_apply_fused_gates(sv_state *st, const sv_fused *f, sv_timing *timings);
 
-/* The launches that a call without timing records makes of f's gates on a complex64 state, in order --
- * host only, no GPU: sv_apply_fused_gates, or (from_basis != 0) sv_init_apply.  Returns their number L
+/* The launches that a call without timing records makes of f's gates on a complex64 state, in order, once
+ * the passes' matrices are uploaded -- host only, no GPU: sv_apply_fused_gates, or (from_basis != 0)
+ * sv_init_apply.  Returns their number L
  * (or a negative SV_E* code) and writes, for the first min(L, max_launches) launches s:
  *   gates[s]        the number of fused gates the launch applies;
  *   on_small[s]     1 when it runs on sv_init_apply's small state;

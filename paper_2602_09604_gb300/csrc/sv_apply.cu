@@ -904,37 +904,51 @@ int make_plan(const sv_fused *f, sv_fused::Plan *pl, const std::vector<char> *la
     return SV_OK;
 }
 
-// The plan of a call, its passes' descriptors and matrices in one device buffer.  Made on the first
-// call of each kind, which waits for this upload but for no work queued on any stream, and kept with f (its gates, their order and the small-state set never change).
-int ensure_plan(sv_fused *f, sv_fused::Plan *pl, const std::vector<char> *lazy, uint64_t A, int a, int device)
+// What a call saves by running a plan's passes as such: microseconds by launch saved.  Measured on a
+// second call (gates of 2, three gates alone / in one pass): 8 to 16 qubits 16 / 13 us, 20 qubits 22 / 20,
+// 22 qubits 39 / 28, 23 qubits 54 / 42, 24 qubits 129 / 78, 26 qubits 477 / 252.
+double plan_saves_us(const sv_fused *f, const sv_fused::Plan &pl, int a)
 {
-    if (pl->ready) return SV_OK;
-    SV_TRY(make_plan(f, pl, lazy, A, a));
+    double us = 0;
+    for (const PassPlan *p : {&pl.small, &pl.rest}) {
+        const int n = p == &pl.small ? a : f->n;
+        for (const PassStep &s : p->steps)
+            if (s.single < 0) us += ((double)s.gates.size() - 1) * (n <= 20 ? 2.0 : n <= 23 ? 5.0 : 12.0);
+    }
+    return us;
+}
+// Taking a buffer for a plan's images and uploading them.  A circuit uploads them in the call in which
+// its calls so far would have saved this much: a long circuit in its first, one of a few gates on a small
+// state in a later one (first call, without / with the upload: two gates on 16 qubits 16 / 23 us, four 21 / 26,
+// eight 28 / 30; two on 20 qubits 18 / 29, two on 23 qubits 35 / 46).
+constexpr double kUploadUs = 12;
+
+// Puts a plan's descriptors and matrices into one device buffer.  Waits for this upload but for no work
+// queued on any stream.
+int upload_plan(sv_fused::Plan *pl, int device)
+{
     const size_t ns = pl->small.image.size(), nr = pl->rest.image.size();
     pl->rest_off = ns;
     const size_t bytes = (ns + nr) * sizeof(float);
-    if (bytes > 0) {
-        const RelaxedCapture relaxed;
-        SharedBuffer *buf = nullptr;
-        SV_TRY(shared_buffer_get(device, bytes, &buf));
-        std::unique_lock<std::mutex> lk;
-        unsigned char *img = nullptr;
-        int rc = pinned_staging(bytes, &img, lk);
-        if (rc == SV_OK) {
-            if (ns) std::memcpy(img, pl->small.image.data(), ns * sizeof(float));
-            if (nr) std::memcpy(img + ns * sizeof(float), pl->rest.image.data(), nr * sizeof(float));
-            rc = upload_now(device, buf->p, img, bytes);
-        }
-        if (rc != SV_OK) {
-            shared_buffer_release(buf);
-            return rc;
-        }
-        pl->buf = buf;
-        pl->d_plan = static_cast<float *>(buf->p);
-        pl->small.image = std::vector<float>();
-        pl->rest.image = std::vector<float>();
+    const RelaxedCapture relaxed;
+    SharedBuffer *buf = nullptr;
+    SV_TRY(shared_buffer_get(device, bytes, &buf));
+    std::unique_lock<std::mutex> lk;
+    unsigned char *img = nullptr;
+    int rc = pinned_staging(bytes, &img, lk);
+    if (rc == SV_OK) {
+        if (ns) std::memcpy(img, pl->small.image.data(), ns * sizeof(float));
+        if (nr) std::memcpy(img + ns * sizeof(float), pl->rest.image.data(), nr * sizeof(float));
+        rc = upload_now(device, buf->p, img, bytes);
     }
-    pl->ready = true;
+    if (rc != SV_OK) {
+        shared_buffer_release(buf);
+        return rc;
+    }
+    pl->buf = buf;
+    pl->d_plan = static_cast<float *>(buf->p);
+    pl->small.image = std::vector<float>();
+    pl->rest.image = std::vector<float>();
     return SV_OK;
 }
 
@@ -1051,30 +1065,45 @@ int apply_core(sv_state *st, sv_fused *f, sv_timing *timings, const std::vector<
         return launch_fused_gate(st->d, st->n, g, device_mats(i), device_tc(i), st->stream, st->num_sms);
     };
     sv_fused::Plan *pl = &f->plans[m > 0 ? 1 : 0];
-    bool planned = !timings && !st->c128;
-    if (planned && (!pl->ready || capturing)) {
-        // The plan's images are uploaded once.  On a stream that is being captured nothing may be
-        // uploaded, and without device memory nothing can be: such a call launches gate by gate.  A
-        // capture that uses them makes its graph one of their owners.
-        planned = capturing ? pl->ready && (!pl->buf || shared_buffer_retain_in_capture(pl->buf, st->stream) == SV_OK)
-                            : ensure_plan(f, pl, m > 0 ? lazy : nullptr, A, a, st->device) == SV_OK;
-        if (!planned) {
+    bool planned = !timings && !st->c128, passes = false;
+    if (planned && !pl->made) {
+        planned = make_plan(f, pl, m > 0 ? lazy : nullptr, A, a) == SV_OK;
+        if (planned) {
+            pl->made = true;
+            pl->saves_us = plan_saves_us(f, *pl, a);
+        }
+    }
+    if (planned && pl->saves_us > 0) {
+        // On a stream that is being captured nothing may be uploaded, and without device memory nothing
+        // can be: such a call launches gate by gate.  A capture that uses the images makes its graph one
+        // of their owners.
+        if (!capturing && !pl->buf) {
+            pl->owed_us += pl->saves_us;
+            if (pl->owed_us >= kUploadUs) upload_plan(pl, st->device);
+        }
+        passes = pl->buf && (!capturing || shared_buffer_retain_in_capture(pl->buf, st->stream) == SV_OK);
+        if (!passes) {
             cudaGetLastError();
             clear_error();
         }
     }
     if (planned) {
-        // no record per gate is asked for: gates go in passes (the plan; see sv_stage.cu)
+        // No record per gate is asked for: gates go in the plan's order, in passes (see sv_stage.cu) or, while
+        // the images are not on the device, one by one with the same result bit by bit.
         for (size_t s = 0; rc == SV_OK && s < pl->small.steps.size(); ++s) {
             const PassStep &ps = pl->small.steps[s];
-            if (ps.single < 0) rc = launch_stage(small, pl->d_plan, ps, st->stream, st->num_sms);
-            else rc = small_gate(pl->small_gates[(size_t)ps.single], (size_t)pl->small_index[(size_t)ps.single]);
+            auto one = [&](int g) { return small_gate(pl->small_gates[(size_t)g], (size_t)pl->small_index[(size_t)g]); };
+            if (ps.single >= 0) rc = one(ps.single);
+            else if (passes) rc = launch_stage(small, pl->d_plan, ps, st->stream, st->num_sms);
+            else for (size_t g = 0; rc == SV_OK && g < ps.gates.size(); ++g) rc = one(ps.gates[g]);
         }
         if (rc == SV_OK && m > 0 && m < ng && !first_reads_small) rc = expand();
         for (size_t s = 0; rc == SV_OK && s < pl->rest.steps.size(); ++s) {
             const PassStep &ps = pl->rest.steps[s];
-            if (ps.single < 0) rc = launch_stage(st->d, pl->d_plan + pl->rest_off, ps, st->stream, st->num_sms);
-            else rc = full_gate((size_t)pl->rest_index[(size_t)ps.single]);
+            auto one = [&](int g) { return full_gate((size_t)pl->rest_index[(size_t)g]); };
+            if (ps.single >= 0) rc = one(ps.single);
+            else if (passes) rc = launch_stage(st->d, pl->d_plan + pl->rest_off, ps, st->stream, st->num_sms);
+            else for (size_t g = 0; rc == SV_OK && g < ps.gates.size(); ++g) rc = one(ps.gates[g]);
         }
     } else {
         for (size_t oi = 0; oi < ng && rc == SV_OK; ++oi) {

@@ -275,12 +275,13 @@ struct sv_fused {
     // launch plans for the calls without timing records, one for sv_apply_fused_gates and one for
     // sv_init_apply (made on first use: the gates, their order and the small-state set are fixed)
     struct Plan {
-        bool ready = false;
+        bool made = false;
+        double saves_us = 0, owed_us = 0;          // what a call saves by its passes; what calls without them would have
         std::vector<svg::FusedGate> small_gates;   // sv_init_apply: the gates of the small state, renumbered
         std::vector<int> small_index, rest_index;  // their and the other gates' indices, in order
         svg::PassPlan small, rest;
         size_t rest_off = 0;                       // floats into d_plan of the second part's image
-        svg::SharedBuffer *buf = nullptr;          // both images, shared with graphs captured from the circuit
+        svg::SharedBuffer *buf = nullptr;          // both images once uploaded, shared with graphs captured from the circuit
         float *d_plan = nullptr;                   // = buf's memory
     };
     Plan plans[2];

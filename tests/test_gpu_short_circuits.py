@@ -1,0 +1,87 @@
+"""Circuits of a few gates: the first calls launch gate by gate, later ones in staged passes (once the
+upload of the passes' matrices has paid), with the same bits; and a first call does not cost an upload
+that it cannot earn back."""
+import statistics
+import time
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2602_09604_gb300 import build as libbuild
+from paper_2602_09604_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    libbuild.build()
+    import torch
+    assert torch.cuda.is_available()
+    from paper_2602_09604_gb300 import binding
+    return binding
+
+
+def circuit(n, k, count, rng):
+    gates = [wl.random_gate(n, int(rng.integers(1, k + 1)), rng) for _ in range(count)]
+    gates.append(wl.Gate((1,), wl.random_unitary(2, rng), tuple(int(q) for q in rng.choice(np.arange(2, n), 5, replace=False))))
+    return gates
+
+
+@pytest.mark.parametrize("lazy", [False, True])
+@pytest.mark.parametrize("n,k,count", [(8, 2, 2), (13, 3, 3), (16, 2, 4), (19, 4, 2), (20, 5, 3), (22, 3, 2), (13, 2, 40), (24, 3, 12)])
+def test_every_call_gives_the_same_bits(B, n, k, count, lazy):
+    import torch
+    from paper_2602_09604_gb300.state import DeviceState
+    rng = np.random.default_rng(n * k + count)
+    gates = circuit(n, k, count, rng)
+    f = B.sv_fuse_circuit(gates, n, max_k=k)
+    st = DeviceState(n)
+    psi = wl.random_state(n, rng).astype(np.complex64)
+    first = None
+    for _ in range(9):
+        if lazy:
+            B.sv_init_apply(st.h, 5, f)
+        else:
+            st.load(psi)
+            st.apply(f)
+        got = st.buf.clone()
+        first = got if first is None else first
+        assert bool((got.view(torch.int32) == first.view(torch.int32)).all())
+    ref = psi.astype(np.complex128)
+    if lazy:
+        ref = oracle.run_circuit(n, gates, 5, threads=oracle.default_threads())
+    else:
+        for g in gates:
+            oracle.apply_gate(ref, n, g, oracle.default_threads())
+    # one fused gate's error on a unit vector is at most (2^(k+1) + 2) 2^-24
+    tol = sum((2 ** (B.sv_fused_get_info(f, i)["k"] + 1) + 2) * 2.0 ** -24 for i in range(B.sv_fused_count(f)))
+    assert oracle.l2_error(ref, st.store()) <= tol
+    B.sv_fused_free(f)
+    st.free()
+
+
+def test_first_calls_of_short_circuits_upload_nothing(B):
+    """Two gates on 16 qubits: first and second calls are the same two launches (15 and 14 us); with an
+    upload in the first it took 1.8 times the second (23 and 13 us)."""
+    import torch
+    from paper_2602_09604_gb300.state import DeviceState
+    n = 16
+    rng = np.random.default_rng(2)
+    gates = [wl.random_gate(n, 2, rng) for _ in range(2)]
+    fused = [B.sv_fuse_circuit(gates, n, mode=B.FUSE_NONE) for _ in range(120)]
+    st = DeviceState(n)
+    st.init(0)
+    torch.cuda.synchronize()
+    times = [[], []]
+    for f in fused:
+        for t in times:
+            began = time.perf_counter()
+            st.apply(f)
+            torch.cuda.synchronize()
+            t.append(time.perf_counter() - began)
+        B.sv_fused_free(f)
+    first, second = (statistics.median(t[20:]) for t in times)
+    assert first < 1.5 * second, (first, second)
+    st.free()
