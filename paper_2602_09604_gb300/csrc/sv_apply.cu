@@ -904,31 +904,37 @@ int make_plan(const sv_fused *f, sv_fused::Plan *pl, const std::vector<char> *la
     return SV_OK;
 }
 
-// What a call saves by running a plan's passes as such: microseconds by launch saved.  Measured on a
-// second call (gates of 2, three gates alone / in one pass): 8 to 16 qubits 16 / 13 us, 20 qubits 22 / 20,
-// 22 qubits 39 / 28, 23 qubits 54 / 42, 24 qubits 129 / 78, 26 qubits 477 / 252.
+// What a call saves by running a plan's passes as such, from the gates' sizes: a share by gate, less one
+// launch.  Measured on a second call (us, alone / in one pass): two gates of 2 on 8 to 16 qubits 14 / 13, six
+// 22 / 14, three on 20 qubits 22 / 20, on 22 qubits 39 / 28, on 24 qubits 129 / 78; eight gates of 4 on 8 to 19
+// qubits 45 / 23, three on 22 qubits 64 / 51; two gates of 5 on 8 qubits 32 / 19, on 12 to 19 qubits
+// 48 / 20, on 22 qubits 88 / 61.
 double plan_saves_us(const sv_fused *f, const sv_fused::Plan &pl, int a)
 {
     double us = 0;
     for (const PassPlan *p : {&pl.small, &pl.rest}) {
-        const int n = p == &pl.small ? a : f->n;
-        for (const PassStep &s : p->steps)
-            if (s.single < 0) us += ((double)s.gates.size() - 1) * (n <= 20 ? 2.0 : n <= 23 ? 5.0 : 12.0);
+        const bool small = p == &pl.small;
+        const int n = small ? a : f->n;
+        const double launch = n >= 24 ? 12 : n >= 21 ? 5 : 2;
+        for (const PassStep &s : p->steps) {
+            if (s.single >= 0) continue;
+            us -= launch;
+            for (int g : s.gates) {
+                const int k = small ? pl.small_gates[(size_t)g].k : f->gates[(size_t)pl.rest_index[(size_t)g]].k;
+                us += k >= 5 ? (n >= 12 ? 15 : 6) : n >= 24 || k <= 3 ? launch : launch + (n >= 21 ? 2 : 1);
+            }
+        }
     }
     return us;
 }
-// Taking a buffer for a plan's images and uploading them.  A circuit uploads them in the call in which
-// its calls so far would have saved this much: a long circuit in its first, one of a few gates on a small
-// state in a later one (first call, without / with the upload: two gates on 16 qubits 16 / 23 us, four 21 / 26,
-// eight 28 / 30; two on 20 qubits 18 / 29, two on 23 qubits 35 / 46).
-constexpr double kUploadUs = 12;
+// What uploading a plan costs: a buffer from the cache, a copy and its end, the images' making.
+double plan_upload_us(const sv_fused::Plan &pl) { return 10 + (double)(pl.small.image_floats + pl.rest.image_floats) / 1024; }
 
-// Puts a plan's descriptors and matrices into one device buffer.  Waits for this upload but for no work
-// queued on any stream.
-int upload_plan(sv_fused::Plan *pl, int device)
+// Makes a plan's images and puts them into one device buffer.  Waits for this upload but for no work queued
+// on any stream.
+int upload_plan(const sv_fused *f, sv_fused::Plan *pl, int a, int device)
 {
-    const size_t ns = pl->small.image.size(), nr = pl->rest.image.size();
-    pl->rest_off = ns;
+    const size_t ns = pl->small.image_floats, nr = pl->rest.image_floats;
     const size_t bytes = (ns + nr) * sizeof(float);
     const RelaxedCapture relaxed;
     SharedBuffer *buf = nullptr;
@@ -937,18 +943,24 @@ int upload_plan(sv_fused::Plan *pl, int device)
     unsigned char *img = nullptr;
     int rc = pinned_staging(bytes, &img, lk);
     if (rc == SV_OK) {
-        if (ns) std::memcpy(img, pl->small.image.data(), ns * sizeof(float));
-        if (nr) std::memcpy(img + ns * sizeof(float), pl->rest.image.data(), nr * sizeof(float));
-        rc = upload_now(device, buf->p, img, bytes);
+        try {
+            std::vector<const FusedGate *> small, rest;
+            for (const FusedGate &g : pl->small_gates) small.push_back(&g);
+            for (int i : pl->rest_index) rest.push_back(&f->gates[(size_t)i]);
+            fill_images(small, a, &pl->small, reinterpret_cast<float *>(img));
+            fill_images(rest, f->n, &pl->rest, reinterpret_cast<float *>(img) + ns);
+            rc = upload_now(device, buf->p, img, bytes);
+        } catch (const std::exception &) {
+            rc = SV_ENOMEM;
+        }
     }
     if (rc != SV_OK) {
         shared_buffer_release(buf);
         return rc;
     }
+    pl->rest_off = ns;
     pl->buf = buf;
     pl->d_plan = static_cast<float *>(buf->p);
-    pl->small.image = std::vector<float>();
-    pl->rest.image = std::vector<float>();
     return SV_OK;
 }
 
@@ -1074,12 +1086,14 @@ int apply_core(sv_state *st, sv_fused *f, sv_timing *timings, const std::vector<
         }
     }
     if (planned && pl->saves_us > 0) {
-        // On a stream that is being captured nothing may be uploaded, and without device memory nothing
-        // can be: such a call launches gate by gate.  A capture that uses the images makes its graph one
-        // of their owners.
+        // A circuit uploads its images in the call in which its calls so far would have saved that cost: a long
+        // one in its first, one of a few gates on a small state in a later one (first call, gates of 2,
+        // without / with the upload: two on 16 qubits 16 / 23 us, four 21 / 26; two on 23 qubits 35 / 46).  On
+        // a stream that is being captured nothing may be uploaded, and without device memory nothing can be.
+        // A capture that uses the images makes its graph one of their owners.
         if (!capturing && !pl->buf) {
             pl->owed_us += pl->saves_us;
-            if (pl->owed_us >= kUploadUs) upload_plan(pl, st->device);
+            if (pl->owed_us >= plan_upload_us(*pl)) upload_plan(f, pl, a, st->device);
         }
         passes = pl->buf && (!capturing || shared_buffer_retain_in_capture(pl->buf, st->stream) == SV_OK);
         if (!passes) {
@@ -1183,11 +1197,16 @@ extern "C" int sv_fused_plan_passes(const sv_fused *f, int from_basis, int max_l
         SV_TRY(make_plan(f, &pl, m > 0 ? &lazy : nullptr, m > 0 ? A : 0, m > 0 ? __builtin_popcountll(A) : 0));
         size_t at = 0, o = 0;
         for (int part = 0; part < 2; ++part) {
-            const PassPlan &p = part ? pl.rest : pl.small;
+            PassPlan &p = part ? pl.rest : pl.small;
             const std::vector<int> &index = part ? pl.rest_index : pl.small_index;
+            std::vector<const FusedGate *> planned;
+            if (part) for (int i : pl.rest_index) planned.push_back(&f->gates[(size_t)i]);
+            else for (const FusedGate &g : pl.small_gates) planned.push_back(&g);
+            std::vector<float> image(p.image_floats);
+            fill_images(planned, part ? f->n : __builtin_popcountll(A), &p, image.data());
             for (const PassStep &s : p.steps) {
                 std::vector<unsigned char> block;
-                if (s.single < 0) pass_block(p, s, &block);
+                if (s.single < 0) pass_block(s, image.data(), &block);
                 if (blocks && at + block.size() <= blocks_bytes) std::memcpy(static_cast<unsigned char *>(blocks) + at, block.data(), block.size());
                 if (launches < max_launches) {
                     if (gates) gates[launches] = s.single < 0 ? (int)s.gates.size() : 1;

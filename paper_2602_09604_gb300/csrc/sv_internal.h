@@ -132,20 +132,22 @@ struct PassStep {
     long long tiles = 0;
     uint64_t tile = 0;          // its local qubits
     std::vector<int> gates;     // what it applies, in order (indices into the planned gates)
-    std::vector<unsigned long long> args;   // the pass's kernel arguments
-    size_t image_off = 0;       // its descriptors and matrices: floats into PassPlan::image
+    std::vector<unsigned long long> args;   // the pass's kernel arguments (fill_images)
+    size_t image_off = 0;       // its descriptors and matrices: floats into the plan's image
 };
 struct PassPlan {
     std::vector<PassStep> steps;
-    std::vector<float> image;   // the passes' descriptors and matrices (16-byte multiples), one after another
+    size_t image_floats = 0;    // the passes' descriptors and matrices (16-byte multiples), one after another
 };
 // Cuts gates (in circuit order, on an n-qubit state) into passes and single launches.  Gates move
 // ahead only of gates on other qubits, and with keep_order not at all: a circuit with a tensor-core
 // gate anywhere keeps its order (the operand split turns a last-bit difference of the input into a
 // larger one).
 void plan_passes(const std::vector<const FusedGate *> &gates, int n, bool keep_order, PassPlan *plan);
+// Writes the passes' images (plan->image_floats floats) and kernel arguments; the gates are those planned.
+void fill_images(const std::vector<const FusedGate *> &gates, int n, PassPlan *plan, float *image);
 // A pass's geometry, descriptors and matrices as they reach its kernel (sv_fused_plan_passes).
-void pass_block(const PassPlan &plan, const PassStep &p, std::vector<unsigned char> *out);
+void pass_block(const PassStep &p, const float *image, std::vector<unsigned char> *out);
 int launch_stage(float *sv, const float *image, const PassStep &p, cudaStream_t stream, int num_sms);
 
 // Tensor-core path (sv_tc.cu): host-side operand images and the launcher.

@@ -270,9 +270,11 @@ uint64_t named(const FusedGate &g)
 
 size_t mat_floats(const FusedGate &g) { return size_t(2) << (2 * g.k); }
 
-// the launch arguments of a pass over gates `idx` with the local qubits `lam` (bits 0-4 set)
-void fill_stage(const std::vector<const FusedGate *> &gates, const std::vector<int> &idx, uint64_t lam, int n, StageArgs *a,
-                std::vector<float> *image)
+constexpr size_t kGateFloats = sizeof(StageGate) / sizeof(float);
+
+// the launch arguments of a pass over gates `idx` with the local qubits `lam` (bits 0-4 set), and its
+// image: descriptors, then matrices
+void fill_stage(const std::vector<const FusedGate *> &gates, const std::vector<int> &idx, uint64_t lam, int n, StageArgs *a, float *image)
 {
     std::memset(a, 0, sizeof(*a));
     int local_of[64];
@@ -281,9 +283,8 @@ void fill_stage(const std::vector<const FusedGate *> &gates, const std::vector<i
         if ((lam >> q) & 1) local_of[q] = L++;
     fill_geom(lam, n, &a->t);
     a->n_gates = (int)idx.size();
-    constexpr size_t kGateFloats = sizeof(StageGate) / sizeof(float);
-    const size_t at0 = image->size();
-    image->resize(at0 + idx.size() * kGateFloats);
+    size_t at = idx.size() * kGateFloats;
+    std::vector<int> free_bits, order;
     for (size_t s = 0; s < idx.size(); ++s) {
         const FusedGate &g = *gates[(size_t)idx[s]];
         StageGate o;
@@ -303,7 +304,7 @@ void fill_stage(const std::vector<const FusedGate *> &gates, const std::vector<i
                     o.cm_out |= uint64_t(1) << q;
                 }
             }
-        std::vector<int> free_bits, order;
+        free_bits.clear();
         for (int t = 0; t < L; ++t)
             if (!((used >> t) & 1)) free_bits.push_back(t);
         lane_bits(free_bits, &order);
@@ -313,19 +314,19 @@ void fill_stage(const std::vector<const FusedGate *> &gates, const std::vector<i
             if (b < 10) o.lane[b % 5] |= b < 5 ? v : v << 16;
             if (b >= 5) o.step[b - 5] = (unsigned short)v;
         }
-        o.moff = (unsigned short)((image->size() - at0) / 4);
+        o.moff = (unsigned short)(at / 4);
         const int D = 1 << g.k;
         for (int j = 0; j < D; ++j)
-            for (int p = 0; p < D / 2; ++p) {
+            for (int p = 0; p < D / 2; ++p, at += 4) {
                 const size_t e0 = size_t(2 * p) * D + j, e1 = e0 + D;
-                image->push_back(g.ur[e0]);
-                image->push_back(g.ur[e1]);
-                image->push_back(g.ui[e0]);
-                image->push_back(g.ui[e1]);
+                image[at] = g.ur[e0];
+                image[at + 1] = g.ur[e1];
+                image[at + 2] = g.ui[e0];
+                image[at + 3] = g.ui[e1];
             }
-        std::memcpy(image->data() + at0 + s * kGateFloats, &o, sizeof(o));
+        std::memcpy(image + s * kGateFloats, &o, sizeof(o));
     }
-    a->units = (int)((image->size() - at0) / 4);
+    a->units = (int)(at / 4);
 }
 
 }  // namespace
@@ -333,7 +334,7 @@ void fill_stage(const std::vector<const FusedGate *> &gates, const std::vector<i
 void plan_passes(const std::vector<const FusedGate *> &gates, int n, bool keep_order, PassPlan *plan)
 {
     plan->steps.clear();
-    plan->image.clear();
+    plan->image_floats = 0;
     const size_t ng = gates.size();
     bool small = true;
     for (const FusedGate *g : gates)
@@ -421,21 +422,29 @@ void plan_passes(const std::vector<const FusedGate *> &gates, int n, bool keep_o
             st.tiles = 1ll << (n - L);
             st.tile = lam;
             st.gates = took;
-            st.image_off = plan->image.size();
-            st.args.assign((sizeof(StageArgs) + 7) / 8, 0);
-            fill_stage(gates, took, lam, n, reinterpret_cast<StageArgs *>(st.args.data()), &plan->image);
+            st.image_off = plan->image_floats;
+            plan->image_floats += took.size() * kGateFloats + mats;
         }
         plan->steps.push_back(std::move(st));
     }
 }
 
-void pass_block(const PassPlan &plan, const PassStep &p, std::vector<unsigned char> *out)
+void fill_images(const std::vector<const FusedGate *> &gates, int n, PassPlan *plan, float *image)
+{
+    for (PassStep &st : plan->steps)
+        if (st.single < 0) {
+            st.args.assign((sizeof(StageArgs) + 7) / 8, 0);
+            fill_stage(gates, st.gates, st.tile, n, reinterpret_cast<StageArgs *>(st.args.data()), image + st.image_off);
+        }
+}
+
+void pass_block(const PassStep &p, const float *image, std::vector<unsigned char> *out)
 {
     const StageArgs *a = reinterpret_cast<const StageArgs *>(p.args.data());
     static_assert(sizeof(StageArgs) == 168, "sv_fused_plan_passes documents the layout");
     out->resize(sizeof(StageArgs) + 16 * (size_t)a->units);
     std::memcpy(out->data(), a, sizeof(StageArgs));
-    std::memcpy(out->data() + sizeof(StageArgs), plan.image.data() + p.image_off, 16 * (size_t)a->units);
+    std::memcpy(out->data() + sizeof(StageArgs), image + p.image_off, 16 * (size_t)a->units);
 }
 
 namespace {

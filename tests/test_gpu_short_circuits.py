@@ -85,3 +85,29 @@ def test_first_calls_of_short_circuits_upload_nothing(B):
     first, second = (statistics.median(t[20:]) for t in times)
     assert first < 1.5 * second, (first, second)
     st.free()
+
+
+def test_first_calls_with_gates_of_five_upload_at_once(B):
+    """Four gates of five qubits on 14 qubits earn the upload in the first call (passes 28 us, gate by gate
+    71): put off by the number of launches alone, the first call took longer than before passes existed."""
+    import torch
+    from paper_2602_09604_gb300.state import DeviceState
+    n = 14
+    rng = np.random.default_rng(5)
+    gates = [wl.random_gate(n, 5, rng, targets=tuple(int(q) for q in rng.choice(9, 5, replace=False))) for _ in range(6)]
+    fused = [B.sv_fuse_circuit(gates, n, mode=B.FUSE_NONE) for _ in range(60)]
+    st = DeviceState(n)
+    st.init(0)
+    torch.cuda.synchronize()
+    times = [[], []]
+    for f in fused:
+        for t in times:
+            began = time.perf_counter()
+            st.apply(f)
+            torch.cuda.synchronize()
+            t.append(time.perf_counter() - began)
+        B.sv_fused_free(f)
+    first, second = (statistics.median(t[10:]) for t in times)
+    # the second call is passes; the first those and an upload, less than the six gates' own launches
+    assert first < 2.2 * second, (first, second)
+    st.free()
