@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(kHighThreads) apply_ctrl_kernel(float *__restr
 }
 
 template <int K>
-int launch_ctrl(float *sv, int n, const FusedGate &g, const float2 *, cudaStream_t stream, int)
+int launch_ctrl(float *sv, int n, const FusedGate &g, const float2 *, cudaStream_t stream, int num_sms)
 {
     CtrlArgs<K> a;
     std::memset(&a, 0, sizeof(a));
@@ -467,7 +467,9 @@ int launch_ctrl(float *sv, int n, const FusedGate &g, const float2 *, cudaStream
     a.cmask = g.cmask;
     a.n_groups = 1ll << (n - np);
     const long long grid = (a.n_groups + kHighThreads - 1) / kHighThreads;
-    return launch_chained(true, apply_ctrl_kernel<K>, (unsigned)grid, kHighThreads, 0, stream, sv, a);
+    // 256 CTAs, six resident on an SM: three targets 5.7 us plain, 7.0 chained (128: 4.6 / 3.8; 512: 7.1 / 6.9)
+    const bool chained = K == 1 || chain_pays(grid, 6ll * num_sms);
+    return launch_chained(chained, apply_ctrl_kernel<K>, (unsigned)grid, kHighThreads, 0, stream, sv, a);
 }
 
 template <int K>
@@ -495,9 +497,10 @@ int launch_high(float *sv, int n, const FusedGate &g, const float2 *umem, cudaSt
             g_occ.high[K] |= bit;
         }
     }
-    (void)num_sms;
     const long long grid = (a.n_items + kHighThreads - 1) / kHighThreads;
-    return launch_chained(true, kern, (unsigned)grid, kHighThreads, smem, stream, sv, a, umem);
+    // gates of up to 3 take 4 us, half of it the launch gap; gates of 6 gain at every size (29.4 us of 32.8)
+    const bool chained = (K != 4 && K != 5) || chain_pays(grid, (long long)high_min_blocks<K>() * num_sms);
+    return launch_chained(chained, kern, (unsigned)grid, kHighThreads, smem, stream, sv, a, umem);
 }
 
 template <int K>
@@ -525,9 +528,12 @@ int launch_tile(float *sv, int n, const FusedGate &g, const float2 *umem, cudaSt
             slot |= bit;
         }
     }
-    (void)num_sms;
     const long long grid = (a.t.n_tiles + kTileWarps - 1) / kTileWarps;
-    return launch_chained(true, kern, (unsigned)grid, kTileThreads, smem, stream, sv, a, umem);
+    // Gates of 5 lose on small grids too (16 qubits, 16 CTAs, mixed: 13.2 us plain, 15.5 chained); short
+    // gates whose tiles are gathered gain in the band (3 qubits, 19 qubits: 5.6 / 4.8), others lose (4.1 / 5.5).
+    const long long resident = (K == 6 ? 2ll : (long long)tile_min_blocks<K>()) * num_sms;   // K = 6: 96 KB of shared memory
+    const bool chained = K == 1 || (K <= 3 && gather) || (K == 5 ? 2 * grid >= resident : chain_pays(grid, resident));
+    return launch_chained(chained, kern, (unsigned)grid, kTileThreads, smem, stream, sv, a, umem);
 }
 
 using LaunchFn = int (*)(float *, int, const FusedGate &, const float2 *, cudaStream_t, int);

@@ -17,6 +17,15 @@ __device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.
 // its first access to the state (at once when the launch before was not of this kind or has ended).
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Whether chaining a one-gate kernel pays at this size: `ctas` of its CTAs, `resident` of which the GPU
+// holds at once.  The next kernel's CTAs take the room that is left, all of it on the SMs with least to
+// do; between a seventh and half of a full GPU they then crowd there while other SMs run dry.  Measured
+// (us a gate in chains of ten, plain / chained), gates of 4: high targets, 19 qubits (64 of 304) 6.2 / 7.0, 18
+// qubits (32) 6.2 / 4.8, 21 qubits (256) 8.7 / 7.7; mixed, 19 qubits (256 of 912) 6.2 / 9.0, 18 qubits
+// (128) 6.2 / 5.0, 20 qubits (512) 8.2 / 7.6; gates of 6, mixed: 19 and 20 qubits (64 and 128 of 304) 24.6 / 30.5
+// and 24.6 / 30.8, 18 qubits (32) 24.6 / 22.2, 21 qubits (256) 34.8 / 31.1.
+inline bool chain_pays(long long ctas, long long resident) { return 7 * ctas <= resident || 2 * ctas >= resident; }
+
 // chained = false: an ordinary launch (the kernel starts when the one before has ended).
 template <typename... P, typename... A>
 int launch_chained(bool chained, void (*kern)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream, A &&...args)

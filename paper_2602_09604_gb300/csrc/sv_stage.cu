@@ -453,7 +453,7 @@ std::mutex g_stage_mu;
 uint64_t g_stage_attr[2][6] = {};   // by form and largest gate: a bit per device
 
 template <int T, int KMAX>
-int launch_form(float *sv, const float *image, const PassStep &p, cudaStream_t stream)
+int launch_form(float *sv, const float *image, const PassStep &p, cudaStream_t stream, int num_sms)
 {
     const StageArgs *a = reinterpret_cast<const StageArgs *>(p.args.data());
     auto kern = stage_kernel<T, KMAX>;
@@ -469,19 +469,23 @@ int launch_form(float *sv, const float *image, const PassStep &p, cudaStream_t s
             slot |= bit;
         }
     }
-    return launch_chained(true, kern, (unsigned)p.tiles, T, (size_t(256) << a->t.fb) + 16 * (size_t)a->units, stream, sv,
+    // A part-filled wave of small CTAs leaves SMs with room, where the next pass's CTAs crowd: with gates of
+    // one or two (five CTAs an SM) 21 qubits, 512 tiles, plain / chained: grid 237 / 259 us, quantum volume
+    // 236 / 251; from 1024 tiles on 408 / 384. Larger gates fill 512 tiles' wave to 0.84 and more: 193 / 170.
+    const bool chained = T == 512 || KMAX > 2 || p.tiles >= (long long)stage_ctas(KMAX) * num_sms;
+    return launch_chained(chained, kern, (unsigned)p.tiles, T, (size_t(256) << a->t.fb) + 16 * (size_t)a->units, stream, sv,
                           reinterpret_cast<const uint4 *>(image), *a);
 }
 
 template <int T>
-int launch_kmax(float *sv, const float *image, const PassStep &p, cudaStream_t stream)
+int launch_kmax(float *sv, const float *image, const PassStep &p, cudaStream_t stream, int num_sms)
 {
     switch (p.kmax) {
     case 1:
-    case 2: return launch_form<T, 2>(sv, image, p, stream);
-    case 3: return launch_form<T, 3>(sv, image, p, stream);
-    case 4: return launch_form<T, 4>(sv, image, p, stream);
-    default: return launch_form<T, 5>(sv, image, p, stream);
+    case 2: return launch_form<T, 2>(sv, image, p, stream, num_sms);
+    case 3: return launch_form<T, 3>(sv, image, p, stream, num_sms);
+    case 4: return launch_form<T, 4>(sv, image, p, stream, num_sms);
+    default: return launch_form<T, 5>(sv, image, p, stream, num_sms);
     }
 }
 
@@ -492,7 +496,8 @@ int launch_stage(float *sv, const float *image, const PassStep &p, cudaStream_t 
     // With few tiles a pass is a chain of short gates, so each tile gets all the threads an SM
     // takes; with many, small CTAs of several groups a thread share an SM and overlap each other's
     // loads, barriers and arithmetic.
-    return p.tiles < 2ll * num_sms ? launch_kmax<512>(sv, image + p.image_off, p, stream) : launch_kmax<128>(sv, image + p.image_off, p, stream);
+    return p.tiles < 2ll * num_sms ? launch_kmax<512>(sv, image + p.image_off, p, stream, num_sms)
+                                      : launch_kmax<128>(sv, image + p.image_off, p, stream, num_sms);
 }
 
 }  // namespace svg

@@ -1241,8 +1241,11 @@ int launch_tc_t(float *sv, int n, const FusedGate &g, const void *dtc, cudaStrea
         a.ph_nb = (n + 7) / 8;
     }
     // Past 2^26 amplitudes a pass takes 160 us and more and there is no launch gap left to win: those
-    // run the plain forms (chained, the staged k = 6 kernel took 3.89 ms instead of 3.69 at 30 qubits).
-    const bool chained = n <= 26 && !vs;
+    // run the plain forms (chained, the staged k = 6 kernel took 3.89 ms instead of 3.69 at 30 qubits).  Two
+    // staged forms lose before (us, plain / chained): 3xBF16 k = 6, 24 qubits 70.6 / 69.9, 25 qubits 129.6 / 131.4,
+    // 26 qubits 245 / 251; k = 5, 25 qubits 114.8 / 114.0, 26 qubits 216.6 / 217.7.
+    const int last_chained = !staged ? 26 : K == 5 ? 25 : K == 6 && MODE == kModeBF16X3 ? 24 : 26;
+    const bool chained = n <= last_chained && !vs;
     VsArgs v{};
     if (vs) v = VsArgs{vs->src, vs->mask, vs->rest, vs->off};
     void (*kern)(float *, const TcArgs) =
