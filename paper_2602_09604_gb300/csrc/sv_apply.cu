@@ -1097,12 +1097,17 @@ int apply_core(sv_state *st, sv_fused *f, sv_timing *timings, const std::vector<
         // without / with the upload: two on 16 qubits 16 / 23 us, four 21 / 26; two on 23 qubits 35 / 46).  On
         // a stream that is being captured nothing may be uploaded, and without device memory nothing can be.
         // A capture that uses the images makes its graph one of their owners.
+        bool failed = false;
         if (!capturing && !pl->buf) {
             pl->owed_us += pl->saves_us;
-            if (pl->owed_us >= plan_upload_us(*pl)) upload_plan(f, pl, a, st->device);
+            if (pl->owed_us >= plan_upload_us(*pl)) failed = upload_plan(f, pl, a, st->device) != SV_OK;
         }
-        passes = pl->buf && (!capturing || shared_buffer_retain_in_capture(pl->buf, st->stream) == SV_OK);
-        if (!passes) {
+        passes = pl->buf != nullptr;
+        if (passes && capturing) {
+            failed = shared_buffer_retain_in_capture(pl->buf, st->stream) != SV_OK;
+            passes = !failed;
+        }
+        if (failed) {   // gate by gate then; a caller's own pending error stays
             cudaGetLastError();
             clear_error();
         }
